@@ -149,6 +149,24 @@ __device__ __forceinline__ bool mbar_wait(uint32_t bar, uint32_t parity, volatil
     }
 }
 
+// One lane of a converged warp: true in exactly one lane, the same one on every call.
+__device__ __forceinline__ bool elect_one() {
+    uint32_t is;
+    asm volatile(
+        "{\n\t.reg .pred p;\n\t"
+        "elect.sync _|p, 0xffffffff;\n\t"
+        "selp.b32 %0, 1, 0, p;\n\t}"
+        : "=r"(is));
+    return is != 0;
+}
+
+// mbar_wait by a whole warp: every lane waits, and all of them learn the same answer
+// from one vote, so the code that follows stays warp-uniform.
+__device__ __forceinline__ bool mbar_wait_warp(uint32_t bar, uint32_t parity, volatile int* abort,
+                                               uint64_t limit_ns = 2000000000ull) {
+    return __all_sync(0xffffffffu, mbar_wait(bar, parity, abort, limit_ns));
+}
+
 // ---- 32-bit shared-memory accesses by address ------------------------------------
 __device__ __forceinline__ void sts_u32(uint32_t addr, uint32_t v) {
     asm volatile("st.shared.u32 [%0], %1;" ::"r"(addr), "r"(v) : "memory");

@@ -26,18 +26,15 @@
 //              one column half per warp).  32-column chunks are read with
 //              tcgen05.ld (the next chunk's load overlaps the current chunk's
 //              work) and reduced with 3-input minima; a chunk is skipped unless
-//              some row of the warp has a key at or below its threshold (the
-//              smaller of the bounds its two column halves have reached).
-//              Survivors (key, column) are stashed in shared memory and, once
-//              the tile's accumulator is back with the MMA warp, appended with
-//              their global ids to the row's candidate pool for that half (in
-//              global memory, no lock: each half has one writer).  A pool that
-//              would overflow is compacted by its warp: a cooperative selection
-//              finds a bound keeping between k' and k' plus an eighth of the
-//              slack entries, the rest are dropped and the threshold lowered.
+//              some row of the warp has a key at or below its threshold.
+//              Survivors (key, column) are appended to the row's candidate pool for
+//              that half (in global memory, no lock: each half has one writer).  A
+//              pool that would overflow is compacted by its warp: a cooperative
+//              selection finds a bound that leaves k' entries or a few more, the
+//              rest are dropped and the row's threshold lowered.
 //              After the sweep k_pool_finalize selects each row's k' smallest
-//              (key, global id) from its two pools, so ties go to the smaller
-//              id whatever the order the candidates came in.
+//              (key, global id) from its two pools, so ties go to the smaller id
+//              whatever the order the candidates came in.
 // Rows are ordered by cell, cells along a chain of nearby pivots (see
 // run_shard_knn), and each sweep starts at the block's own tile and moves
 // outward, so the thresholds are tight after the first few tiles and later
@@ -68,13 +65,15 @@ constexpr int KB8 = 128;                // 8-bit elements per 128-byte K block
 constexpr int KAUG = 16;                // norm block: 16 elements (32 bytes)
 constexpr int A_BLK_BYTES = BM * 128;   // one K block of the 128 A rows
 constexpr int A_AUG_BYTES = BM * 32;
-constexpr int NAUG = 1;                 // norm-block slots (loaded first in each tile)
+constexpr int NAUG = 2;                 // norm-block slots (loaded first in each tile)
 constexpr int NACC = 2;
 constexpr int EPI_WARPS = 8;            // two warps per TMEM lane quarter
-constexpr int PH_MAX = 320;             // candidate pool entries per row half, at most
-constexpr int SC = 24;                  // survivors a thread stashes before a tile's release
-constexpr int KS = 33;                  // floats per row of a warp's key scratch (32 + 1 pad)
-constexpr int THREADS = 64 + 32 * EPI_WARPS;
+constexpr int PH_MAX = 384;             // candidate pool entries per row half, at most
+constexpr int EPI_WARP0 = 4;            // first epilogue warp (whole warpgroups: setmaxnreg)
+constexpr int THREADS = 32 * (EPI_WARP0 + EPI_WARPS);
+// Registers per thread after the split: 168 x 384 at launch; 40 x 128 + 224 x 256 =
+// 62,464 <= 64,512 after it.
+constexpr int REGS_ISSUE = 40, REGS_EPI = 224;
 constexpr uint32_t TMEM_COLS = NACC * BNMAX;
 constexpr int MAX_NST = 6;
 constexpr int CELL = 128;               // rows per pivot cell, short rows (at most 1024 a shard)
@@ -104,12 +103,24 @@ enum TileCounter {
     TC_MMA_ISSUE,        // MMA thread: cycles issuing tcgen05.mma
     TC_MMA_COMMIT,       // MMA thread: cycles in tcgen05.commit
     TC_MMA_LOOP,         // MMA thread: cycles from the A wait to the end of the tile loop
-    TC_STASH,            // epilogue threads: cycles writing survivors to the stash
-    TC_DIRECT,           // epilogue threads: cycles appending a chunk straight to the pools
-    TC_FLUSH_LOOP,       // epilogue threads: cycles moving stashed survivors to the pools
+    TC_STASH,            // (unused: 0)
+    TC_DIRECT,           // epilogue threads: cycles storing a chunk's survivors to the pools
+    TC_FLUSH_LOOP,       // (unused: 0)
     TC_N
 };
 __device__ unsigned long long g_tile_counters[TC_N];
+
+// Global operand scale from the largest |x| (float bits): E4M3 maps it to 448 (the
+// largest finite value); scaled FP16 multiplies by the power of two that puts it in
+// [2^13, 2^14) (exact, and far from both overflow and the subnormal range).
+__device__ __forceinline__ float operand_scale(unsigned int amax_bits, bool e4m3) {
+    const float am = __uint_as_float(amax_bits);
+    if (!(am > 0.0f && am <= 3.0e38f)) return 1.0f;
+    if (e4m3) return 448.0f / am;
+    int ex;
+    frexpf(am, &ex);
+    return ldexpf(1.0f, 14 - ex);
+}
 
 struct KnnParams {
     const int64_t* blk_off;  // [nprob+1] prefix sums of row blocks
@@ -136,7 +147,7 @@ struct KnnParams {
     int ksteps, hs;
     uint32_t idesc_neg, idesc_aug;
     uint32_t* out_id;
-    float* out_d;
+    float* out_d;  // NULL: ids only (the lists are re-ranked)
     int* status;
     // Exact tile skipping (NULL: every tile of the row block's shard).  tlist:
     // TL_MAX entries per row block, the column tiles it sweeps in sweep order;
@@ -145,30 +156,39 @@ struct KnnParams {
     const uint16_t* tlist;
     const int* tcount;
     // Candidate pools (global memory): A row a, column half h holds its survivors
-    // at pool[(2 a + h) * ph ...], their number in pool_cnt[2 a + h] after the sweep.
+    // at pool[(2 a + h) * ph ...] as (key bits << 32 | column of the problem), their
+    // number in pool_cnt[2 a + h] after the sweep.  k' = 1: one entry per half, order
+    // bits of the key << 32 | global id (or all ones).
     uint64_t* pool;
     int* pool_cnt;
     int ph;
     // Optional upper bound of every A row's k'-th squared distance (rowub[a]; NULL:
     // none): the sweep starts with that threshold.  Keys of split operands carry an
-    // error, covered by the relative margin ub_margin (0 for exact keys).
+    // error, covered by the relative margin ub_margin (0 for exact keys); keys of
+    // scaled FP16 operands carry the square of the operand scale, a power of two made
+    // from *ub_amax (NULL: no scale).
     const float* rowub;
     float ub_margin;
+    const unsigned int* ub_amax;
 };
 
 // Entries of a row half's candidate pool, whole warps: 256 (what a compaction holds
-// in registers) for list widths 32 to 128, the list width plus 64 above; always at
-// least 32 more than k' (a chunk's survivors fit after a compaction).  A larger pool
-// compacts less often at the same cost per compaction.
-__host__ __device__ inline int pool_half(int kprime) {
+// in registers) for list widths 32 to 128, the list width plus 64 above, and a quarter
+// of the list width more where the lists are re-ranked (the memory that the screened
+// distances would take, which nothing reads: with k' = 256 a compaction of 384 entries
+// frees 120 of them, of 320 only 56); always at least 32 more than k' (a chunk's
+// survivors fit after a compaction).  A larger pool compacts less often at about the
+// same cost per compaction.
+__host__ __device__ inline int pool_half(int kprime, bool rerank) {
     int ph = kprime < 32 ? 2 * kprime : kprime <= 128 ? 256 : kprime + 64;
     if (ph < kprime + 32) ph = kprime + 32;
     ph = (ph + 31) / 32 * 32;
+    if (rerank && kprime > 128) ph += kprime / 4 / 32 * 32;
     return ph > kt::PH_MAX ? kt::PH_MAX : ph;
 }
 
 struct KnnSmemLayout {
-    uint32_t a, aaug, b, baug, tau, stash, kscr, bars, tmem_slot, abort_flag, total;
+    uint32_t a, aaug, b, baug, tau, kscr, bars, tmem_slot, abort_flag, total;
 };
 
 // a_stream = 0: the CTA's A rows stay resident (nkb_a K blocks) and a ring stage
@@ -190,12 +210,10 @@ __host__ __device__ inline KnnSmemLayout knn_smem_layout(int bn, int nkb_a, int 
     o += nst * knn_stage_bytes(bn, a_stream);
     L.baug = o;
     o += kt::NAUG * bn * 32;
-    L.tau = o;  // [2][BM] floats: each column half's current k'-th key per row
-    o += 2 * kt::BM * 4;
-    L.stash = o;  // [EPI_WARPS][SC][32] survivors (key bits << 32 | column), lane-minor
-    o += kt::EPI_WARPS * kt::SC * 32 * 8;
-    L.kscr = o;   // [EPI_WARPS][32][KS] a chunk's keys, one row per thread
-    o += kt::EPI_WARPS * 32 * kt::KS * 4;
+    L.tau = o;  // [BM] threshold of each row (order bits), [2][BM] each half's bound
+    o += 3 * kt::BM * 4;
+    L.kscr = o;   // [EPI_WARPS][32][32] a chunk's keys, one row per thread (swizzled)
+    o += kt::EPI_WARPS * 32 * 32 * 4;
     L.bars = o;
     o += (2 * kt::MAX_NST + 2 * kt::NAUG + 2 * kt::NACC + 2) * 8;
     L.tmem_slot = o;
@@ -247,143 +265,99 @@ __device__ __forceinline__ float min32(const float (&k)[32]) {
 }
 
 // ---- per-row candidate pools ----------------------------------------------------
-// The smallest `kp` composite values (key bits << 32 | global id) among a warp's
-// entries, E per lane (UINT64_MAX = no entry), n valid in all: returns the kp-th
-// smallest valid value (the largest valid one when n <= kp).  Bisection first on
-// the key bits, then on the ids of the entries tied at the k-th key; every count is
-// a warp-wide sum (redux.sync), so all lanes return the same value.
-template <int E>
-__device__ __forceinline__ uint64_t warp_select_kth(const uint64_t (&v)[E], int n, int kp) {
-    const uint32_t FULL = 0xffffffffu;
-    uint32_t kmin = 0xFFFFFFFFu, kmax = 0;
-#pragma unroll
-    for (int e = 0; e < E; ++e) {
-        if (v[e] != ~0ull) {
-            const uint32_t h = (uint32_t)(v[e] >> 32);
-            kmin = h < kmin ? h : kmin;
-            kmax = h > kmax ? h : kmax;
-        }
-    }
-    kmin = __reduce_min_sync(FULL, kmin);
-    kmax = __reduce_max_sync(FULL, kmax);
-    if (n <= kp) {  // every entry stays: the largest one
-        uint32_t imax = 0;
-#pragma unroll
-        for (int e = 0; e < E; ++e)
-            if (v[e] != ~0ull && (uint32_t)(v[e] >> 32) == kmax) {
-                const uint32_t id = (uint32_t)v[e];
-                imax = id > imax ? id : imax;
-            }
-        imax = __reduce_max_sync(FULL, imax);
-        return ((uint64_t)kmax << 32) | imax;
-    }
-    // least key K with #{key <= K} >= kp: each step counts at three pivots that
-    // split [lo, hi] in four (independent warp sums) and keeps one quarter
-    uint32_t lo = kmin, hi = kmax;
-    while (lo < hi) {
-        const uint32_t q = (hi - lo) >> 2;
-        const uint32_t p1 = lo + q, p2 = lo + ((hi - lo) >> 1), p3 = hi - q - 1 > p2 ? hi - q - 1 : p2;
-        uint32_t c1 = 0, c2 = 0, c3 = 0;
-#pragma unroll
-        for (int e = 0; e < E; ++e) {
-            const uint32_t h = (uint32_t)(v[e] >> 32);
-            c1 += h <= p1 ? 1u : 0u;
-            c2 += h <= p2 ? 1u : 0u;
-            c3 += h <= p3 ? 1u : 0u;
-        }
-        c1 = __reduce_add_sync(FULL, c1);
-        c2 = __reduce_add_sync(FULL, c2);
-        c3 = __reduce_add_sync(FULL, c3);
-        if (c1 >= (uint32_t)kp) hi = p1;
-        else if (c2 >= (uint32_t)kp) { lo = p1 + 1; hi = p2; }
-        else if (c3 >= (uint32_t)kp) { lo = p2 + 1; hi = p3; }
-        else lo = p3 + 1;
-    }
-    const uint32_t K = lo;
-    uint32_t below = 0, tied = 0, imin = 0xFFFFFFFFu, imax = 0;
-#pragma unroll
-    for (int e = 0; e < E; ++e) {
-        const uint32_t h = (uint32_t)(v[e] >> 32), id = (uint32_t)v[e];
-        below += h < K ? 1u : 0u;
-        if (h == K && v[e] != ~0ull) {
-            ++tied;
-            imin = id < imin ? id : imin;
-            imax = id > imax ? id : imax;
-        }
-    }
-    below = __reduce_add_sync(FULL, below);
-    tied = __reduce_add_sync(FULL, tied);
-    imin = __reduce_min_sync(FULL, imin);
-    imax = __reduce_max_sync(FULL, imax);
-    const uint32_t need = (uint32_t)kp - below;  // 1 <= need <= tied
-    if (need >= tied) return ((uint64_t)K << 32) | imax;
-    uint32_t ilo = imin, ihi = imax;  // least id I with #{key == K, id <= I} >= need
-    while (ilo < ihi) {
-        const uint32_t mid = ilo + ((ihi - ilo) >> 1);
-        uint32_t c = 0;
-#pragma unroll
-        for (int e = 0; e < E; ++e)
-            c += ((uint32_t)(v[e] >> 32) == K && v[e] != ~0ull && (uint32_t)v[e] <= mid) ? 1u : 0u;
-        c = __reduce_add_sync(FULL, c);
-        if (c >= need) ihi = mid; else ilo = mid + 1;
-    }
-    return ((uint64_t)K << 32) | ilo;
+// A pool entry is (key bits << 32 | shard column), the key as its float bits; loaded
+// for a selection it becomes (order bits of the key << 32 | column), UINT64_MAX = no
+// entry.  Global ids are looked up (column_gid) only where they decide: for entries
+// tied at the boundary key, and for the entries a row ends up with.
+__device__ __forceinline__ uint64_t pool_load(const uint64_t* p) {
+    const uint64_t x = *p;
+    return ((uint64_t)f2ord(__uint_as_float((uint32_t)(x >> 32))) << 32) | (uint32_t)x;
+}
+__device__ __forceinline__ uint64_t pool_raw(uint64_t v) {
+    return ((uint64_t)__float_as_uint(ord2f((uint32_t)(v >> 32))) << 32) | (uint32_t)v;
+}
+__device__ __forceinline__ uint32_t column_gid(const uint32_t* gidrow, uint32_t col) {
+    return gidrow ? __ldg(gidrow + col) : col;
 }
 
-// A bound T with kp <= #{entries <= T} <= maxkeep (n > maxkeep valid entries, E per
-// lane): the same search on the key bits as warp_select_kth, stopped as soon as the
-// keys at or below the upper end of the range number at most maxkeep; only when
-// more than maxkeep entries share the kp-th key are the ids of those entries
-// searched (then exactly kp stay).  Every entry at or below T is kept by the
-// caller, so the bound tightens by whole keys without an exact selection.
+// What a selection keeps: entries with key < key, and those with key == key whose
+// global id is at most id (id = 0xFFFFFFFF: all of them).
+struct Bound {
+    uint32_t key, id;
+};
+__device__ __forceinline__ bool bound_keeps(const Bound& T, uint64_t v, const uint32_t* gidrow) {
+    const uint32_t h = (uint32_t)(v >> 32);
+    if (v == ~0ull || h > T.key) return false;
+    if (h < T.key || T.id == 0xFFFFFFFFu) return true;
+    return column_gid(gidrow, (uint32_t)v) <= T.id;
+}
+
+// A bound that keeps between kp and maxkeep of a warp's n <= 640 entries (E per lane;
+// n > maxkeep >= kp), exactly kp when maxkeep == kp.  Each step counts the keys at or
+// below three pivots (10 bits each of one warp sum, so all lanes return the same
+// value): two around the place where the wanted rank falls if the keys between lo and
+// hi are spread evenly, one in the middle of what lies above.  It stops as soon as the
+// keys at or below a pivot number kp to maxkeep: two or three steps for spread keys,
+// where halving the range of the key bits takes nine or more.  Only when more than
+// maxkeep entries share the kp-th key are their global ids searched (then exactly kp
+// stay).
 template <int E>
-__device__ __forceinline__ uint64_t warp_select_bound(const uint64_t (&v)[E], int n, int kp,
-                                                      int maxkeep) {
+__device__ __forceinline__ Bound warp_select(const uint64_t (&v)[E], int n, int kp, int maxkeep,
+                                             const uint32_t* gidrow) {
     const uint32_t FULL = 0xffffffffu;
     uint32_t kmin = 0xFFFFFFFFu, kmax = 0;
 #pragma unroll
     for (int e = 0; e < E; ++e) {
-        if (v[e] != ~0ull) {
-            const uint32_t h = (uint32_t)(v[e] >> 32);
-            kmin = h < kmin ? h : kmin;
-            kmax = h > kmax ? h : kmax;
-        }
+        const uint32_t h = (uint32_t)(v[e] >> 32);
+        kmin = h < kmin ? h : kmin;
+        kmax = v[e] != ~0ull && h > kmax ? h : kmax;
     }
     kmin = __reduce_min_sync(FULL, kmin);
     kmax = __reduce_max_sync(FULL, kmax);
-    // invariant: #{key <= hi} = chi >= kp, #{key < lo} < kp
-    uint32_t lo = kmin, hi = kmax, chi = (uint32_t)n;
-    while (chi > (uint32_t)maxkeep && lo < hi) {
-        const uint32_t q = (hi - lo) >> 2;
-        const uint32_t p1 = lo + q, p2 = lo + ((hi - lo) >> 1), p3 = hi - q - 1 > p2 ? hi - q - 1 : p2;
-        uint32_t c1 = 0, c2 = 0, c3 = 0;
+    // invariant: #{key <= hi} = chi >= kp, #{key < lo} = clo < kp
+    uint32_t lo = kmin, hi = kmax;
+    int chi = n, clo = 0;
+    while (chi > maxkeep && lo < hi) {
+        // pivots lie in [lo, hi); interpolated on the key values (on their bits a range
+        // across zero is exponential), the last one halves the bits that are left, so
+        // every step makes progress
+        const float f = (0.5f * (float)(kp + maxkeep) - (float)clo) / (float)(chi - clo);
+        const float flo = ord2f(lo), fw = ord2f(hi) - flo;
+        uint32_t p1 = f2ord(fmaf(0.8f * f, fw, flo)), p2 = f2ord(fmaf(1.2f * f, fw, flo));
+        p1 = p1 < lo ? lo : p1 > hi - 1 ? hi - 1 : p1;
+        p2 = p2 < p1 ? p1 : p2 > hi - 1 ? hi - 1 : p2;
+        const uint32_t p3 = hi - 1 - ((hi - 1 - p2) >> 1);
+        uint32_t c = 0;
 #pragma unroll
         for (int e = 0; e < E; ++e) {
             const uint32_t h = (uint32_t)(v[e] >> 32);
-            c1 += h <= p1 ? 1u : 0u;
-            c2 += h <= p2 ? 1u : 0u;
-            c3 += h <= p3 ? 1u : 0u;
+            c += (h <= p1 ? 1u : 0u) + (h <= p2 ? 1u << 10 : 0u) + (h <= p3 ? 1u << 20 : 0u);
         }
-        c1 = __reduce_add_sync(FULL, c1);
-        c2 = __reduce_add_sync(FULL, c2);
-        c3 = __reduce_add_sync(FULL, c3);
-        if (c1 >= (uint32_t)kp) { hi = p1; chi = c1; }
-        else if (c2 >= (uint32_t)kp) { lo = p1 + 1; hi = p2; chi = c2; }
-        else if (c3 >= (uint32_t)kp) { lo = p2 + 1; hi = p3; chi = c3; }
-        else lo = p3 + 1;
+        c = __reduce_add_sync(FULL, c);
+        const int c1 = c & 1023, c2 = (c >> 10) & 1023, c3 = c >> 20;
+        if (c1 >= kp) { hi = p1; chi = c1; }
+        else if (c2 >= kp) { lo = p1 + 1; clo = c1; hi = p2; chi = c2; }
+        else if (c3 >= kp) { lo = p2 + 1; clo = c2; hi = p3; chi = c3; }
+        else { lo = p3 + 1; clo = c3; }
     }
-    if (chi <= (uint32_t)maxkeep) return ((uint64_t)hi << 32) | 0xFFFFFFFFull;
+    Bound T;
+    T.key = hi;
+    T.id = 0xFFFFFFFFu;
+    if (chi <= maxkeep) return T;
     // more than maxkeep entries at or below the kp-th key K = hi: the ties at K are
-    // split by id so that exactly kp entries stay
+    // split by global id so that exactly kp entries stay
     const uint32_t K = hi;
     uint32_t below = 0, imin = 0xFFFFFFFFu, imax = 0;
+    uint32_t id[E];
 #pragma unroll
     for (int e = 0; e < E; ++e) {
-        const uint32_t h = (uint32_t)(v[e] >> 32), id = (uint32_t)v[e];
+        const uint32_t h = (uint32_t)(v[e] >> 32);
         below += h < K ? 1u : 0u;
+        id[e] = 0xFFFFFFFFu;
         if (h == K && v[e] != ~0ull) {
-            imin = id < imin ? id : imin;
-            imax = id > imax ? id : imax;
+            id[e] = column_gid(gidrow, (uint32_t)v[e]);
+            imin = id[e] < imin ? id[e] : imin;
+            imax = id[e] > imax ? id[e] : imax;
         }
     }
     below = __reduce_add_sync(FULL, below);
@@ -396,161 +370,111 @@ __device__ __forceinline__ uint64_t warp_select_bound(const uint64_t (&v)[E], in
         uint32_t c = 0;
 #pragma unroll
         for (int e = 0; e < E; ++e)
-            c += ((uint32_t)(v[e] >> 32) == K && v[e] != ~0ull && (uint32_t)v[e] <= mid) ? 1u : 0u;
+            c += ((uint32_t)(v[e] >> 32) == K && v[e] != ~0ull && id[e] <= mid) ? 1u : 0u;
         c = __reduce_add_sync(FULL, c);
         if (c >= need) ihi = mid; else ilo = mid + 1;
     }
-    return ((uint64_t)K << 32) | ilo;
+    T.id = ilo;
+    return T;
 }
 
-// Per-row top-k state of one epilogue thread (lane = row, one column half).
-// Survivors of the threshold test are appended to the row half's pool in global
-// memory (no lock: each half has its own pool); a pool about to overflow is
-// compacted by the whole warp to its kp smallest entries, which makes the kp-th
-// of them the half's new threshold tau.  A column half's entries above the other
-// half's tau cannot be among the row's kp smallest either, so the test uses
-// teff = min(tau, other half's tau) (read from shared memory; it only decreases,
-// so a stale value is still a valid bound).  With kp = 1 the pool is the running
-// minimum in a register.
+// State of one epilogue thread (lane = row, one column half).  thr is the row's
+// threshold (order bits in shared memory, lowered by either half; it only decreases, so
+// a stale copy is still a valid bound): a half's own k'-th key or, for wide lists, the
+// larger of two published bounds q, each with at least ceil(k'/2) of its half's keys
+// at or below it, so that k' keys of the row lie at or below the larger one (near the
+// row's k'-th key, where a half's k'-th is near the row's 2k'-th).  With kp = 1 there
+// is no pool but a running minimum in a register.
 struct EpiState {
-    uint64_t* pool;       // this thread's row half
-    uint64_t* pool0;      // row 0 of the warp, same half (row r at pool0 + 2 r ph)
-    float* tau_own;       // shared [BM]: this half's tau per row
-    const volatile float* tau_other;
-    uint64_t* stash;      // shared: this warp's stash, entry e of lane l at [e * 32 + l]
+    uint64_t* pool0;      // row 0 of the warp, this half (row r at pool0 + 2 r ph)
+    uint32_t* thr;        // shared, threshold of the warp's 32 rows (order bits)
+    volatile float* q_own;    // shared, this half's bounds of the warp's 32 rows
+    volatile float* q_other;  // the other half's
     const uint32_t* gidrow;  // global id of each column of the shard (NULL: the column)
-    uint32_t kscr;        // shared address of this thread's row of the key scratch
-    int row, kp, ph, c, sn;
-    float tau, teff;
+    uint32_t kscr;        // shared address of this thread's row of the warp's key scratch
+    int kp, ph, c;
+    float teff;
     uint64_t best;        // kp == 1
     // counters (used only by the profiling instantiation)
     unsigned long long c_flush_cyc, c_chunks, c_slow, c_flushes, c_iters, c_app;
-    unsigned long long c_ldw, c_filter, c_append, c_stash, c_direct, c_floop;
+    unsigned long long c_ldw, c_filter, c_append, c_direct;
 };
+__device__ __forceinline__ float row_threshold(const uint32_t* thr) {
+    return ord2f(*(const volatile uint32_t*)thr);
+}
 
-// Compact the pools of the rows in `mask` (lanes of this warp) to their kp
-// smallest entries and lower those rows' tau.  Each lane passes its row's count
-// and tau and gets them back (changed only for the rows compacted).  Kept out of
-// line: it is rare, and the sweep loop keeps two chunks of keys in registers.
-struct PoolState {
-    int c;
-    float tau;
-};
+// Compact the pools of the rows in `mask` (lanes of this warp) and lower those rows'
+// thresholds; s.c is the lane's own row's count.  Entries above the row's threshold go;
+// where that would leave more than maxkeep (the other half's bound is missing or
+// loose), the half keeps its kp smallest or a few more.  Inlined: a called function
+// would be given the registers of the issuing warps.
 template <int EM>  // EM * 32 >= ph
-__device__ __noinline__ PoolState epi_compact(uint64_t* pool0, int ph, int kp, int c, float tau,
-                                              uint32_t mask, float* tau_own, int row) {
-    __syncwarp();  // every lane's appends are visible to the warp
+__device__ __forceinline__ void epi_compact(EpiState& s, uint32_t mask) {
     const int lane = threadIdx.x & 31;
-    const int E = ph >> 5;
+    // a part of the slack may stay above the wanted rank, which lets a search stop early
+    const int kh = (s.kp + 1) >> 1;
+    int maxkeep = s.kp + ((s.ph - s.kp) >> 3);
+    if (maxkeep > s.ph - 32) maxkeep = s.ph - 32;
+    const int maxhalf = kh + ((maxkeep - kh) >> 3);
+    // The halves' bounds cost a second search while one of them is missing: worth it
+    // where keeping k' entries would free less than half of the pool (k' >= 128;
+    // measured at k' = 256: 27.0 -> 22.5 ms, 128: 77.9 -> 73.8 ms, but 80: 72.2 -> 75.3).
+    const bool halves = 2 * s.kp >= s.ph;
+    __syncwarp();  // every lane's appends are visible to the warp
     while (mask) {
         const int r = __ffs(mask) - 1;
         mask &= mask - 1;
-        const int cr = __shfl_sync(0xffffffffu, c, r);
-        uint64_t* pr = pool0 + (int64_t)r * 2 * ph;
+        const int cr = __shfl_sync(0xffffffffu, s.c, r);
+        if (cr <= maxkeep) continue;
+        uint64_t* pr = s.pool0 + (int64_t)r * 2 * s.ph;
         uint64_t v[EM];
 #pragma unroll
         for (int e = 0; e < EM; ++e) {
             const int idx = lane + 32 * e;
-            v[e] = (e < E && idx < cr) ? pr[idx] : ~0ull;
+            v[e] = idx < cr ? pool_load(pr + idx) : ~0ull;
         }
-        // keep between kp and maxkeep entries: an eighth of the slack may stay
-        // above the kp-th, which lets the bound stop early
-        int maxkeep = kp + ((ph - kp) >> 3);
-        if (maxkeep > ph - 32) maxkeep = ph - 32;
-        if (maxkeep < kp) maxkeep = kp;
-        const uint64_t T = cr > maxkeep ? warp_select_bound(v, cr, kp, maxkeep) : ~0ull - 1;
+        Bound T;
+        for (int want = halves ? kh : s.kp, most = halves ? maxhalf : maxkeep;;) {
+            T = warp_select(v, cr, want, most, s.gidrow);
+            if (want == s.kp) break;
+            const float own = fminf(ord2f(T.key), s.q_own[r]);
+            const uint32_t t = f2ord(fmaxf(own, s.q_other[r]));
+            int n = 0;
+#pragma unroll
+            for (int e = 0; e < EM; ++e) n += (uint32_t)(v[e] >> 32) <= t && v[e] != ~0ull;
+            n = __reduce_add_sync(0xffffffffu, n);
+            __syncwarp();
+            if (lane == 0) s.q_own[r] = own;
+            if (n <= maxkeep) {
+                T.key = t;
+                T.id = 0xFFFFFFFFu;
+                break;
+            }
+            want = s.kp;
+            most = maxkeep;
+        }
         __syncwarp();  // every load done before the pool is rewritten in place
         int base = 0;
 #pragma unroll
         for (int e = 0; e < EM; ++e) {
-            const bool keep = v[e] <= T && v[e] != ~0ull;
+            const bool keep = bound_keeps(T, v[e], s.gidrow);
             const uint32_t b = __ballot_sync(0xffffffffu, keep);
-            if (keep) pr[base + __popc(b & ((1u << lane) - 1u))] = v[e];
+            if (keep) pr[base + __popc(b & ((1u << lane) - 1u))] = pool_raw(v[e]);
             base += __popc(b);
         }
-        __syncwarp();
-        if (lane == r) {
-            c = base;
-            if (cr > maxkeep) {
-                tau = fminf(tau, ord2f((uint32_t)(T >> 32)));
-                tau_own[row] = tau;
-            }
-        }
+        if (lane == 0) atomicMin(s.thr + r, T.key);
+        if (lane == r) s.c = base;
     }
     __syncwarp();
-    PoolState o;
-    o.c = c;
-    o.tau = tau;
-    return o;
-}
-
-// Compact the pools of the rows whose count would pass ph with `add` more entries.
-template <bool PROF, int EMX>
-__device__ __forceinline__ void epi_make_room(EpiState& s, int add) {
-    const uint32_t over = __ballot_sync(0xffffffffu, s.c + add > s.ph);
-    if (over) {
-        long long t0 = 0;
-        if (PROF) t0 = clock64();
-        // one call site: a dispatch on ph here costs the sweep loop registers
-        const PoolState o =
-            epi_compact<EMX>(s.pool0, s.ph, s.kp, s.c, s.tau, over, s.tau_own, s.row);
-        s.c = o.c;
-        s.tau = o.tau;
-        s.teff = fminf(s.tau, s.tau_other[s.row]);
-        if (PROF) {
-            s.c_flush_cyc += clock64() - t0;
-            ++s.c_flushes;
-            s.c_iters += __popc(over);
-        }
-    }
-}
-
-// Move every thread's stashed survivors (key bits << 32 | shard column) into its
-// pool as (key bits << 32 | global id), after a tile's accumulator is released.
-template <bool PROF, int EMX>
-__device__ __forceinline__ void epi_flush_stash(EpiState& s) {
-    if (!__any_sync(0xffffffffu, s.sn > 0)) return;
-    long long f0 = 0;
-    if (PROF) f0 = clock64();
-    epi_make_room<PROF, EMX>(s, s.sn);
-    long long fl0 = 0;
-    if (PROF) fl0 = clock64();
-    const int lane = threadIdx.x & 31;
-    const int mx = __reduce_max_sync(0xffffffffu, (uint32_t)s.sn);
-    for (int e0 = 0; e0 < mx; e0 += 4) {
-        uint64_t v[4];
-        uint32_t g[4];
-#pragma unroll
-        for (int q = 0; q < 4; ++q) v[q] = e0 + q < s.sn ? s.stash[(e0 + q) * 32 + lane] : ~0ull;
-#pragma unroll
-        for (int q = 0; q < 4; ++q) {
-            const uint32_t col = (uint32_t)v[q];
-            g[q] = (v[q] != ~0ull && s.gidrow) ? __ldg(s.gidrow + col) : col;
-        }
-#pragma unroll
-        for (int q = 0; q < 4; ++q) {
-            if (v[q] != ~0ull && ord2f((uint32_t)(v[q] >> 32)) <= s.teff) {
-                s.pool[s.c] = (v[q] & 0xFFFFFFFF00000000ull) | g[q];
-                ++s.c;
-                if (PROF) ++s.c_app;
-            }
-        }
-    }
-    s.sn = 0;
-    __syncwarp();
-    if (PROF) {
-        const long long f1 = clock64();
-        s.c_floop += f1 - fl0;
-        s.c_append += f1 - f0;
-    }
 }
 
 // One 32-column chunk: keys come straight from TMEM; masked columns become NaN
-// (every comparison with NaN is false, and the minimum skips NaN).  A chunk with
-// survivors stashes them (shared memory, no global id yet) so the accumulator can
-// go back to the MMA warp soon; a thread whose stash cannot take them has the
-// stashes emptied first, and a chunk with more survivors than a stash holds (the
-// first tiles of a sweep) goes straight to the pools.
+// (every comparison with NaN is false, and the minimum skips NaN).  In a chunk with
+// survivors each thread marks its own, lays its keys out in the warp's scratch (8
+// stores of 16 bytes; the 16-byte groups of row r are permuted by r & 7, so the
+// stores hit distinct banks) and copies the marked ones to its pool: a loop as long
+// as the busiest lane's count, with nothing looked up and nothing waited for (the
+// entry holds the column; unrolled per-column code ran slower than the work it did).
 template <bool PROF, int EMX>
 __device__ __forceinline__ void epi_chunk(EpiState& s, const uint32_t (&v)[32], int j0, int i,
                                           int n_cols, int self_exclude, bool edge) {
@@ -590,66 +514,49 @@ __device__ __forceinline__ void epi_chunk(EpiState& s, const uint32_t (&v)[32], 
             if (key[u] <= s.teff && x < s.best) s.best = x;
         }
         if (s.best != ~0ull) {
-            s.tau = ord2f((uint32_t)(s.best >> 32));
-            s.teff = s.tau;
+            s.teff = ord2f((uint32_t)(s.best >> 32));
         }
         if (PROF) s.c_append += clock64() - f0;
         return;
     }
-    s.teff = fminf(s.tau, s.tau_other[s.row]);
+    s.teff = row_threshold(s.thr + lane);
     uint32_t surv = 0;  // bit u: column j0 + u survives for this row
 #pragma unroll
     for (int u = 0; u < 32; ++u) surv |= (key[u] <= s.teff ? 1u : 0u) << u;
-    if (__any_sync(0xffffffffu, s.sn + __popc(surv) > kt::SC)) {
-        epi_flush_stash<PROF, EMX>(s);
-        surv = 0;
+    if (!__any_sync(0xffffffffu, surv != 0)) return;
+    long long d0 = 0;
+    if (PROF) d0 = clock64();
+    const uint32_t sw = lane & 7;
 #pragma unroll
-        for (int u = 0; u < 32; ++u) surv |= (key[u] <= s.teff ? 1u : 0u) << u;
-        if (__any_sync(0xffffffffu, __popc(surv) > kt::SC)) {
-            // straight to the pools, global ids shuffled from the lanes that hold them
-            uint32_t g_l = (uint32_t)(j0 + lane);
-            if (s.gidrow && j0 + lane < n_cols) g_l = __ldg(s.gidrow + j0 + lane);
-            epi_make_room<PROF, EMX>(s, __popc(surv));
-            long long d0 = 0;
-            if (PROF) d0 = clock64();
-            const uint32_t any_col = __reduce_or_sync(0xffffffffu, surv);
-#pragma unroll
-            for (int u = 0; u < 32; ++u) {
-                if ((any_col >> u) & 1u) {
-                    const uint32_t gid = __shfl_sync(0xffffffffu, g_l, u);
-                    if (key[u] <= s.teff) {
-                        s.pool[s.c] = ((uint64_t)f2ord(key[u]) << 32) | gid;
-                        ++s.c;
-                        if (PROF) ++s.c_app;
-                    }
-                }
-            }
-            if (PROF) {
-                const long long f1 = clock64();
-                s.c_direct += f1 - d0;
-                s.c_append += f1 - f0;
-            }
-            return;
+    for (int g = 0; g < 8; ++g)
+        asm volatile("st.shared.v4.f32 [%0], {%1, %2, %3, %4};" ::"r"(s.kscr + ((g ^ sw) << 4)),
+                     "f"(key[4 * g]), "f"(key[4 * g + 1]), "f"(key[4 * g + 2]), "f"(key[4 * g + 3])
+                     : "memory");
+    // (each thread reads back only what it stored)
+    const int n = __popc(surv);
+    const uint32_t over = __ballot_sync(0xffffffffu, n && s.c + n > s.ph);
+    if (over) {
+        long long t0 = 0;
+        if (PROF) t0 = clock64();
+        epi_compact<EMX>(s, over);
+        if (PROF) {
+            s.c_flush_cyc += clock64() - t0;
+            ++s.c_flushes;
+            s.c_iters += __popc(over);
         }
     }
-    long long w0 = 0;
-    if (PROF) w0 = clock64();
-    // the chunk's keys to this thread's scratch row (a fixed number of stores, rows
-    // padded so the warp's stores hit distinct banks), then only the survivors
-    // into the stash (a loop as long as the thread's survivor count)
-    if (surv) {
-#pragma unroll
-        for (int u = 0; u < 32; ++u) sts_u32(s.kscr + 4 * u, v[u]);
-        for (uint32_t m = surv; m; m &= m - 1) {
-            const int u = __ffs(m) - 1;
-            const float kv = __uint_as_float(lds_u32(s.kscr + 4 * u));
-            s.stash[s.sn * 32 + lane] = ((uint64_t)f2ord(kv) << 32) | (uint32_t)(j0 + u);
-            ++s.sn;
-        }
+    uint2* dst = (uint2*)(s.pool0 + (int64_t)lane * 2 * s.ph) + s.c;
+    s.c += n;
+    for (uint32_t w = surv; w; w &= w - 1) {
+        const uint32_t u = __ffs(w) - 1;
+        const uint32_t kb = lds_u32(s.kscr + (((u >> 2) ^ sw) << 4) + (u & 3) * 4);
+        *dst++ = make_uint2((uint32_t)j0 + u, kb);
     }
+    __syncwarp();
     if (PROF) {
+        s.c_app += n;
         const long long f1 = clock64();
-        s.c_stash += f1 - w0;
+        s.c_direct += f1 - d0;
         s.c_append += f1 - f0;
     }
 }
@@ -687,8 +594,7 @@ __device__ __forceinline__ int tile_at(int tt, int t0, int ntiles) {
 }
 
 // EMX: pool entries per row half / 32 that the compaction holds in registers
-// (ph <= 32 EMX); a larger EMX costs the sweep loop registers, so the common
-// pools (ph <= 256) use their own instantiation.
+// (ph <= 32 EMX); the common pools (ph <= 256) use their own instantiation.
 template <int BN, bool PROF, int EMX>
 __global__ void __launch_bounds__(kt::THREADS, 1)
     k_knn_tiles(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUtensorMap tmB,
@@ -739,7 +645,9 @@ __global__ void __launch_bounds__(kt::THREADS, 1)
     volatile uint32_t* tmem_slot = (volatile uint32_t*)(base + L.tmem_slot);
     volatile int* abort_flag = (volatile int*)(base + L.abort_flag);
 
-    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    // (the broadcast tells the compiler that the warp index is warp-uniform)
+    const int warp = __shfl_sync(0xffffffffu, (int)(threadIdx.x >> 5), 0);
+    const int lane = threadIdx.x & 31;
     long long cta_t0 = 0;
     if (PROF) cta_t0 = clock64();
     if (threadIdx.x == 0) {
@@ -764,27 +672,37 @@ __global__ void __launch_bounds__(kt::THREADS, 1)
         tmem_alloc(smem_u32((const void*)tmem_slot), kt::TMEM_COLS);
         tmem_relinquish();
     }
-    if (warp >= 2) {  // thresholds of both column halves: the window bound, or +inf
-        const int q = warp & 3, h = (warp - 2) >> 2;
-        const int row = q * 32 + lane;
+    if (warp >= kt::EPI_WARP0 && warp < kt::EPI_WARP0 + 4) {  // thresholds: the window bound, or +inf
+        const int row = (warp & 3) * 32 + lane;
         const int i = rb * kt::BM + row;
         float t = INFINITY;
         if (P.rowub && i < pr.n_rows) {
-            const float ub = P.rowub[pr.a_row0 + i];
+            float ub = P.rowub[pr.a_row0 + i];
             if (ub < INFINITY) {
-                // key = (dist - |x|^2) / 2, rounded up; split keys get the margin
+                if (P.ub_amax) {
+                    const float sc = operand_scale(*P.ub_amax, false);
+                    ub = __fmul_ru(__fmul_ru(ub, sc), sc);
+                }
+                // key = (dist - |x|^2) / 2, rounded up; keys with an error get the margin
                 const float nx = P.na[pr.a_row0 + i];
                 const float d = __fmaf_ru(P.ub_margin, 3.0f * nx + 2.0f * ub, ub);
-                t = 0.5f * __fsub_ru(d, nx);
+                if (d < INFINITY) t = 0.5f * __fsub_ru(d, nx);
             }
         }
-        ((float*)(base + L.tau))[h * kt::BM + row] = t;
+        ((uint32_t*)(base + L.tau))[row] = f2ord(t);
+        ((float*)(base + L.tau))[kt::BM + row] = INFINITY;
+        ((float*)(base + L.tau))[2 * kt::BM + row] = INFINITY;
     }
     tc_fence_before();
     __syncthreads();
     tc_fence_after();
     const uint32_t tmem = *tmem_slot;
 
+    // The epilogue holds two chunks of keys beside its state: with the 168 registers of
+    // an even split its spills (over 100 bytes a thread) do not fit the L1 that 227 KB
+    // of shared memory leave, and every reload costs an L2 access.
+    if (warp < kt::EPI_WARP0) {
+    asm volatile("setmaxnreg.dec.sync.aligned.u32 %0;" ::"n"(kt::REGS_ISSUE));
     if (warp == 0) {
         // ------------------------------------------------------------ producer
         if (lane == 0) {
@@ -855,43 +773,53 @@ __global__ void __launch_bounds__(kt::THREADS, 1)
         }
     } else if (warp == 1) {
         // ------------------------------------------------------------- MMA
-        if (lane == 0) {
-            bool ok = mbar_wait(a_bar, 0, abort_flag);
+        // The whole warp walks the loop and takes every wait (one vote each), and one
+        // elected lane issues: tcgen05.mma takes its descriptors from uniform
+        // registers, and under a plain "lane == 0" branch they are not known to be
+        // uniform, which cost about 258 cycles an MMA whatever its width (128 x 256 x 16
+        // takes 128): 1,121 ns a tile of 9 MMAs without any epilogue, 969 now that the
+        // wait is for the operands (12 KB an MMA read and 8 KB written through the
+        // shared memory's 128 bytes a clock).
+        bool ok = mbar_wait_warp(a_bar, 0, abort_flag);
+        tc_fence_after();
+        int st = 0, sa = 0;
+        uint32_t ph = 0, aph = 0;
+        const int H2 = P.nkb_b >> 1;
+        unsigned long long w_full = 0, w_acc = 0, c_iss = 0, c_com = 0;
+        long long loop0 = 0;
+        if (PROF) loop0 = clock64();
+        for (int t = 0; t < nrun && ok; ++t) {
+            const int a = t % kt::NACC;
+            long long w0 = 0;
+            if (PROF) w0 = clock64();
+            ok = mbar_wait_warp(acce_bar + 8 * a, ((t / kt::NACC) & 1) ^ 1, abort_flag);
+            if (!ok) break;
+            if (PROF) w_acc += clock64() - w0;
             tc_fence_after();
-            int st = 0, sa = 0;
-            uint32_t ph = 0, aph = 0;
-            const int H2 = P.nkb_b >> 1;
-            unsigned long long w_full = 0, w_acc = 0, c_iss = 0, c_com = 0;
-            long long loop0 = 0;
-            if (PROF) loop0 = clock64();
-            for (int t = 0; t < nrun && ok; ++t) {
-                const int a = t % kt::NACC;
-                long long w0 = 0;
-                if (PROF) w0 = clock64();
-                if (!mbar_wait(acce_bar + 8 * a, ((t / kt::NACC) & 1) ^ 1, abort_flag)) {
-                    ok = false;
-                    break;
-                }
-                if (PROF) w_acc += clock64() - w0;
-                tc_fence_after();
-                const uint32_t d_tmem = tmem + a * BN;
-                // D = [1,1,1,0..] . [h,m,l,0..] (= |y|^2 / 2), then D -= x . y
-                if (PROF) w0 = clock64();
-                if (!mbar_wait(afull_bar + 8 * sa, aph, abort_flag)) { ok = false; break; }
-                if (PROF) w_full += clock64() - w0;
-                tc_fence_after();
+            const uint32_t d_tmem = tmem + a * BN;
+            // D = [1,1,1,0..] . [h,m,l,0..] (= |y|^2 / 2), then D -= x . y
+            if (PROF) w0 = clock64();
+            ok = mbar_wait_warp(afull_bar + 8 * sa, aph, abort_flag);
+            if (!ok) break;
+            if (PROF) w_full += clock64() - w0;
+            tc_fence_after();
+            if (elect_one()) {
                 umma_f16(d_tmem, sdesc_sw32(sAaug), sdesc_sw32(sBaug + sa * B_AUG_BYTES),
                          P.idesc_aug, 0);
                 umma_commit(aempty_bar + 8 * sa);
-                if (++sa == kt::NAUG) { sa = 0; aph ^= 1; }
-                const uint32_t accum = 1;
-                for (int j = 0; j < P.nkb_b; ++j) {
-                    if (PROF) w0 = clock64();
-                    if (!mbar_wait(full_bar + 8 * st, ph, abort_flag)) { ok = false; break; }
-                    if (PROF) w_full += clock64() - w0;
-                    tc_fence_after();
-                    if (PROF) w0 = clock64();
-                    const uint32_t bsm = sB + st * STG;
+            }
+            __syncwarp();
+            if (++sa == kt::NAUG) { sa = 0; aph ^= 1; }
+            const uint32_t accum = 1;
+            for (int j = 0; j < P.nkb_b; ++j) {
+                if (PROF) w0 = clock64();
+                ok = mbar_wait_warp(full_bar + 8 * st, ph, abort_flag);
+                if (!ok) break;
+                if (PROF) w_full += clock64() - w0;
+                tc_fence_after();
+                if (PROF) w0 = clock64();
+                const uint32_t bsm = sB + st * STG;
+                if (elect_one()) {
                     if (P.mode == 1 && !P.a_stream) {
                         // compact split sections (A resident): B step sb < hs (hi)
                         // meets A steps sb (hi . hi) and sb + hs (lo . hi); B step
@@ -912,16 +840,14 @@ __global__ void __launch_bounds__(kt::THREADS, 1)
                             }
                         }
                     } else {
-                        int ablk[2];
-                        int na = 1;
-                        if (P.mode == 0) {
-                            ablk[0] = j;
-                        } else if (j < H2) {
-                            ablk[0] = j;       // hi . hi
-                            ablk[1] = H2 + j;  // lo . hi
-                            na = 2;
-                        } else {
-                            ablk[0] = j - H2;  // hi . lo
+                        int ablk0 = j, ablk1 = 0, na = 1;
+                        if (P.mode != 0) {
+                            if (j < H2) {
+                                ablk1 = H2 + j;  // hi . hi, then lo . hi
+                                na = 2;
+                            } else {
+                                ablk0 = j - H2;  // hi . lo
+                            }
                         }
                         // K steps of the block that hold data: the last block of plain
                         // operands may end in zero steps, which are not issued
@@ -929,7 +855,7 @@ __global__ void __launch_bounds__(kt::THREADS, 1)
                         for (int q = 0; q < na; ++q) {
                             const uint32_t asm_ = P.a_stream
                                                       ? bsm + B_BLK_BYTES + q * kt::A_BLK_BYTES
-                                                      : sA + ablk[q] * kt::A_BLK_BYTES;
+                                                      : sA + (q ? ablk1 : ablk0) * kt::A_BLK_BYTES;
                             // four K steps of 32 bytes per 128-byte block (K = 16 for
                             // 16-bit operands, K = 32 for E4M3)
                             if (full) {
@@ -954,59 +880,56 @@ __global__ void __launch_bounds__(kt::THREADS, 1)
                             }
                         }
                     }
-                    long long w1 = 0;
-                    if (PROF) {
-                        w1 = clock64();
-                        c_iss += w1 - w0;
-                    }
                     umma_commit(empty_bar + 8 * st);
-                    if (PROF) c_com += clock64() - w1;
-                    if (++st == P.nst) { st = 0; ph ^= 1; }
                 }
-                if (!ok) break;
-                umma_commit(accf_bar + 8 * a);
+                __syncwarp();
+                if (PROF) c_iss += clock64() - w0;
+                if (++st == P.nst) { st = 0; ph ^= 1; }
             }
+            if (!ok) break;
+            if (elect_one()) umma_commit(accf_bar + 8 * a);
+            __syncwarp();
+        }
+        // every issued MMA completes before TMEM is released
+        if (elect_one()) umma_commit(done_bar);
+        __syncwarp();
+        int dummy = 0;
+        mbar_wait_warp(done_bar, 0, &dummy, 200000000ull);
+        if (lane == 0) {
+            if (!ok) atomicOr(P.status, DEV_TIMEOUT);
             if (PROF) {
                 prof_add(TC_MMA_LOOP, (unsigned long long)(clock64() - loop0));
                 prof_add(TC_MMA_ISSUE, c_iss);
                 prof_add(TC_MMA_COMMIT, c_com);
-            }
-            umma_commit(done_bar);  // every issued MMA completes before TMEM is released
-            int dummy = 0;
-            mbar_wait(done_bar, 0, &dummy, 200000000ull);
-            if (!ok) atomicOr(P.status, DEV_TIMEOUT);
-            if (PROF) {
                 prof_add(TC_MMA_WAIT_FULL, w_full);
                 prof_add(TC_MMA_WAIT_ACC, w_acc);
             }
         }
+    }
     } else {
+        asm volatile("setmaxnreg.inc.sync.aligned.u32 %0;" ::"n"(kt::REGS_EPI));
         // -------------------------------------------------------- epilogue
         // Warp (q, h): TMEM lane quarter q (rows 32q..32q+31), columns
         // [128h, 128h + 128) of every tile.
         const int q = warp & 3;
-        const int h = (warp - 2) >> 2;
+        const int h = (warp - kt::EPI_WARP0) >> 2;
         EpiState s;
-        s.row = q * 32 + lane;
-        const int i = rb * kt::BM + s.row;     // row index inside the problem
-        const int i0 = rb * kt::BM + q * 32;   // first row of this warp
-        const int64_t arow0 = pr.a_row0 + i0;  // gathered A row of lane 0
+        const int i = rb * kt::BM + q * 32 + lane;  // row index inside the problem
+        const int i0 = rb * kt::BM + q * 32;        // first row of this warp
+        const int64_t arow0 = pr.a_row0 + i0;       // gathered A row of lane 0
         s.ph = P.ph;
+        s.c = 0;
         s.kp = P.kprime;
         s.pool0 = P.pool + (arow0 * 2 + h) * (int64_t)P.ph;
-        s.pool = s.pool0 + (int64_t)lane * 2 * P.ph;
-        s.tau_own = (float*)(base + L.tau) + h * kt::BM;
-        s.tau_other = (const volatile float*)((float*)(base + L.tau) + (1 - h) * kt::BM);
-        s.c = 0;
-        s.sn = 0;
-        s.stash = (uint64_t*)(base + L.stash) + (warp - 2) * kt::SC * 32;
-        s.kscr = smem_u32(base + L.kscr) + ((warp - 2) * 32 + lane) * kt::KS * 4;
+        s.thr = (uint32_t*)(base + L.tau) + q * 32;
+        s.q_own = (volatile float*)(base + L.tau) + (1 + h) * kt::BM + q * 32;
+        s.q_other = (volatile float*)(base + L.tau) + (2 - h) * kt::BM + q * 32;
+        s.kscr = smem_u32(base + L.kscr) + ((warp - kt::EPI_WARP0) * 32 + lane) * 128;
         s.gidrow = P.gid ? P.gid + pr.b_row0 : nullptr;
         s.best = ~0ull;
-        s.tau = s.tau_own[s.row];
-        s.teff = fminf(s.tau, s.tau_other[s.row]);
+        s.teff = row_threshold(s.thr + lane);
         s.c_flush_cyc = s.c_chunks = s.c_slow = s.c_flushes = s.c_iters = s.c_app = 0;
-        s.c_ldw = s.c_filter = s.c_append = s.c_stash = s.c_direct = s.c_floop = 0;
+        s.c_ldw = s.c_filter = s.c_append = s.c_direct = 0;
         unsigned long long e_wait = 0;
         long long e_t0 = 0;
         if (PROF) e_t0 = clock64();
@@ -1020,7 +943,11 @@ __global__ void __launch_bounds__(kt::THREADS, 1)
             ++run;
             long long w0 = 0;
             if (PROF) w0 = clock64();
-            if (!mbar_wait(accf_bar + 8 * a, par, abort_flag)) { ok = false; break; }
+            // one lane polls: 32 lanes of eight warps polling take the shared-memory
+            // pipe from the others (Deep-like shards 90.9 -> 86.2 ms in one variant)
+            int there = 1;
+            if (lane == 0) there = mbar_wait(accf_bar + 8 * a, par, abort_flag);
+            if (!__shfl_sync(0xffffffffu, there, 0)) { ok = false; break; }
             if (PROF) e_wait += clock64() - w0;
             tc_fence_after();
             {
@@ -1059,12 +986,8 @@ __global__ void __launch_bounds__(kt::THREADS, 1)
                                         edge);
                     __syncwarp();
                 }
-                // the accumulator is back with the MMA warp: the tile's stashed
-                // survivors join the pools while the next tile is computed
-                epi_flush_stash<PROF, EMX>(s);
             }
         }
-        ok = __all_sync(0xffffffffu, ok);
         if (PROF) {
             prof_add_warp(TC_EPI_CYCLES, (unsigned long long)(clock64() - e_t0));
             prof_add_warp(TC_EPI_WAIT, e_wait);
@@ -1073,9 +996,7 @@ __global__ void __launch_bounds__(kt::THREADS, 1)
             prof_add_warp(TC_LD_WAIT, s.c_ldw);
             prof_add_warp(TC_FILTER, s.c_filter);
             prof_add_warp(TC_APPEND, s.c_append);
-            prof_add_warp(TC_STASH, s.c_stash);
             prof_add_warp(TC_DIRECT, s.c_direct);
-            prof_add_warp(TC_FLUSH_LOOP, s.c_floop);
             if (lane == 0) {
                 prof_add(TC_CHUNKS, s.c_chunks);
                 prof_add(TC_SLOW_CHUNKS, s.c_slow);
@@ -1084,14 +1005,16 @@ __global__ void __launch_bounds__(kt::THREADS, 1)
             }
         }
         if (!ok || *abort_flag) {
+            *abort_flag = 1;
             if (lane == 0) atomicOr(P.status, DEV_TIMEOUT);
-        } else if (i < pr.n_rows) {
-            // the pool's size (k_pool_finalize merges the two halves)
-            if (s.kp == 1) {
-                if (s.best != ~0ull) s.pool[0] = s.best;
-                s.c = s.best != ~0ull ? 1 : 0;
-            }
-            P.pool_cnt[(pr.a_row0 + i) * 2 + h] = s.c;
+        }
+        // the pool's size, none after an abort (k' = 1: this half's smallest;
+        // k_pool_finalize1 takes the smaller of the two)
+        if (i < pr.n_rows) {
+            if (s.kp == 1)
+                s.pool0[(int64_t)lane * 2 * s.ph] = s.best;
+            else
+                P.pool_cnt[(pr.a_row0 + i) * 2 + h] = ok ? s.c : 0;
         }
     }
     tc_fence_before();
@@ -1228,22 +1151,7 @@ __global__ void k_gather(const void* X, int dtype, int d, const int64_t* __restr
                          int64_t rows_cap, int mode, int Kp, int Kh, T* __restrict__ G,
                          float* __restrict__ norms, __nv_bfloat16* __restrict__ aug,
                          const unsigned int* __restrict__ amax_bits) {
-    // Global operand scale: E4M3 maps max|x| to 448 (the largest finite value);
-    // scaled FP16 multiplies by the power of two that puts max|x| in [2^13, 2^14)
-    // (exact, and far from both overflow and the subnormal range).
-    float scale = 1.0f;
-    if (amax_bits) {
-        const float am = __uint_as_float(*amax_bits);
-        if (am > 0.0f && am <= 3.0e38f) {
-            if (sizeof(T) == 1) {
-                scale = 448.0f / am;
-            } else {
-                int ex;
-                frexpf(am, &ex);
-                scale = ldexpf(1.0f, 14 - ex);
-            }
-        }
-    }
+    const float scale = amax_bits ? operand_scale(*amax_bits, sizeof(T) == 1) : 1.0f;
     const int lane = threadIdx.x & 31;
     const int64_t warp_g = (blockIdx.x * (int64_t)blockDim.x + threadIdx.x) >> 5;
     const int64_t nwarps = ((int64_t)gridDim.x * blockDim.x) >> 5;
@@ -1622,9 +1530,9 @@ __device__ __forceinline__ void warp_bitonic_u64(uint64_t (&v)[E]) {
 // Every valid A row of the tile launch's problems: the kprime smallest entries of
 // the union of its two column halves' pools, sorted by (key, global id), written as
 // (global id, |x|^2 + 2 key) to the first k_out slots of its output row, then ANN_PAD
-// / +inf.  One warp per row: the row's entries are selected with warp_select_kth,
-// gathered into shared memory in ballot order, then sorted with a warp bitonic sort
-// of KE entries per lane.
+// / +inf.  One warp per row: the row's entries are selected with warp_select, the
+// kept ones take their global ids and are gathered into shared memory in ballot
+// order, then sorted with a warp bitonic sort of KE entries per lane.
 template <int KE, int EH>  // KE: sorted entries per lane; EH = ph / 32
 __global__ void __launch_bounds__(256)
 k_pool_finalize(const KnnParams P) {
@@ -1639,12 +1547,12 @@ k_pool_finalize(const KnnParams P) {
     const KnnProblem pr = P.probs[lo];
     const int rb = (int)(bid - P.blk_off[lo]);
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const uint32_t* gidrow = P.gid ? P.gid + pr.b_row0 : nullptr;
     uint64_t* stg = stage[warp];
     for (int r = warp; r < kt::BM; r += 8) {
         const int i = rb * kt::BM + r;
         if (i >= pr.n_rows) break;
         const int64_t arow = pr.a_row0 + i;
-        // counts clamped to the pool (an aborted sweep leaves them unwritten)
         const int c0 = min(max(P.pool_cnt[arow * 2], 0), P.ph);
         const int c1 = min(max(P.pool_cnt[arow * 2 + 1], 0), P.ph);
         const uint64_t* h0 = P.pool + arow * 2 * (int64_t)P.ph;
@@ -1653,19 +1561,21 @@ k_pool_finalize(const KnnParams P) {
 #pragma unroll
         for (int e = 0; e < EH; ++e) {
             const int idx = lane + 32 * e;
-            v[e] = idx < c0 ? h0[idx] : ~0ull;
-            v[EH + e] = idx < c1 ? h1[idx] : ~0ull;
+            v[e] = idx < c0 ? pool_load(h0 + idx) : ~0ull;
+            v[EH + e] = idx < c1 ? pool_load(h1 + idx) : ~0ull;
         }
         const int n = c0 + c1;
         const int kp = P.kprime;
-        const uint64_t T = n > 0 ? warp_select_kth(v, n, kp) : 0ull;
+        Bound T;
+        T.key = T.id = 0xFFFFFFFFu;
+        if (n > kp) T = warp_select(v, n, kp, kp, gidrow);
         // the kept entries (kp of them, or all n) into the staging array
         for (int e = lane; e < 32 * KE; e += 32) stg[e] = ~0ull;
         __syncwarp();
         int base = 0;
 #pragma unroll
         for (int e = 0; e < 2 * EH; ++e) {
-            const bool keep = n > 0 && v[e] != ~0ull && v[e] <= T;
+            const bool keep = bound_keeps(T, v[e], gidrow);
             const uint32_t b = __ballot_sync(0xffffffffu, keep);
             const int pos = base + __popc(b & ((1u << lane) - 1u));
             if (keep && pos < 32 * KE) stg[pos] = v[e];
@@ -1674,7 +1584,11 @@ k_pool_finalize(const KnnParams P) {
         __syncwarp();
         uint64_t w[KE];
 #pragma unroll
-        for (int e = 0; e < KE; ++e) w[e] = stg[lane * KE + e];
+        for (int e = 0; e < KE; ++e) {
+            w[e] = stg[lane * KE + e];
+            if (w[e] != ~0ull)
+                w[e] = (w[e] & 0xFFFFFFFF00000000ull) | column_gid(gidrow, (uint32_t)w[e]);
+        }
         __syncwarp();
         warp_bitonic_u64<KE>(w);
         const float nx = P.na[arow];
@@ -1690,7 +1604,7 @@ k_pool_finalize(const KnnParams P) {
                     dd = fmaf(2.0f, ord2f((uint32_t)(w[e] >> 32)), nx);
                 }
                 P.out_id[orow * P.k_out + slot] = id;
-                P.out_d[orow * P.k_out + slot] = dd;
+                if (P.out_d) P.out_d[orow * P.k_out + slot] = dd;
             }
         }
     }
@@ -1711,8 +1625,8 @@ __global__ void __launch_bounds__(kt::BM) k_pool_finalize1(const KnnParams P) {
     if (i >= pr.n_rows) return;
     const int64_t arow = pr.a_row0 + i;
     const uint64_t* h0 = P.pool + arow * 2 * (int64_t)P.ph;
-    const uint64_t a = P.pool_cnt[arow * 2] > 0 ? h0[0] : ~0ull;
-    const uint64_t b = P.pool_cnt[arow * 2 + 1] > 0 ? h0[P.ph] : ~0ull;
+    const uint64_t a = h0[0];
+    const uint64_t b = h0[P.ph];
     const uint64_t w = a < b ? a : b;
     const int64_t orow = P.outrow ? P.outrow[arow] : pr.out_row0 + i;
     uint32_t id = ANN_PAD;
@@ -2606,8 +2520,7 @@ size_t knn_ws(int C, int64_t rows, const KnnPlan& pl, KnnWs* out, void* base, si
     w.ones = cv.take<__nv_bfloat16>((size_t)128 * kt::KAUG);
     w.norms = cv.take<float>((size_t)w.rows_cap + 512);
     w.cand_id = pl.rerank ? cv.take<uint32_t>((size_t)rows * pl.kprime) : nullptr;
-    w.cand_d = pl.rerank ? cv.take<float>((size_t)rows * pl.kprime) : nullptr;
-    w.pool = cv.take<uint64_t>((size_t)w.rows_cap * 2 * pool_half(pl.kprime));
+    w.pool = cv.take<uint64_t>((size_t)w.rows_cap * 2 * pool_half(pl.kprime, pl.rerank));
     w.pool_cnt = cv.take<int>((size_t)w.rows_cap * 2);
     w.src = cv.take<int64_t>((size_t)w.rows_cap);
     w.gid = cv.take<uint32_t>((size_t)w.rows_cap);
@@ -2716,6 +2629,7 @@ static int launch_tiles(const KnnPlan& pl, const void* GA, int64_t rowsA, const 
     ANN_FINALIZE(8, 8)
     ANN_FINALIZE(8, 9)
     ANN_FINALIZE(8, 10)
+    ANN_FINALIZE(8, 12)
 #undef ANN_FINALIZE
     return fail(ANN_ERR_UNSUPPORTED, "tile launch: no finalize for k' = %d, pool %d", P.kprime,
                 P.ph);
@@ -2803,9 +2717,10 @@ static KnnParams base_params(const KnnPlan& pl, int k, const int64_t* blk_off,
     P.tcount = nullptr;
     P.pool = nullptr;
     P.pool_cnt = nullptr;
-    P.ph = pool_half(pl.kprime);
+    P.ph = pool_half(pl.kprime, pl.rerank);
     P.rowub = nullptr;
     P.ub_margin = 0.0f;
+    P.ub_amax = nullptr;
     return P;
 }
 
@@ -2883,16 +2798,7 @@ static int side_stream(cudaStream_t* s, cudaEvent_t* fork_ev, cudaEvent_t* join_
 // square of the operand scale (448 / max|x| for E4M3, a power of two for FP16).
 __global__ void k_unscale_dist(float* __restrict__ dist, int64_t n, const unsigned int* amax_bits,
                                int e4m3) {
-    const float am = __uint_as_float(*amax_bits);
-    if (!(am > 0.0f && am <= 3.0e38f)) return;
-    float scale;
-    if (e4m3) {
-        scale = 448.0f / am;
-    } else {
-        int ex;
-        frexpf(am, &ex);
-        scale = ldexpf(1.0f, 14 - ex);
-    }
+    const float scale = operand_scale(*amax_bits, e4m3 != 0);
     const float inv = 1.0f / scale;
     for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < n;
          i += (int64_t)gridDim.x * blockDim.x)
@@ -2975,7 +2881,7 @@ int run_shard_knn(const void* X, int64_t N, int d, int dtype, const uint32_t* me
     // 3. the kNN sweep
     const bool to_cand = pl.rerank && !screen_only;
     KnnParams P = base_params(pl, k, w.blk_off, w.probs, C, w.norms, w.gid, w.outrow, 1, 1,
-                              to_cand ? w.cand_id : knn_id, to_cand ? w.cand_d : knn_d);
+                              to_cand ? w.cand_id : knn_id, to_cand ? nullptr : knn_d);
     P.pool = w.pool;
     P.pool_cnt = w.pool_cnt;
     const int64_t grid = rows / kt::BM + C + 1;
@@ -3038,9 +2944,9 @@ int run_shard_knn(const void* X, int64_t N, int d, int dtype, const uint32_t* me
         ANN_CHECK_LAUNCH();
         P.tlist = w.tlist;
         P.tcount = w.tcount;
-        // each row's window bound starts its threshold (keys in the data's units:
-        // not for scaled operands, whose keys carry the square of the scale)
-        P.rowub = pl.scaled ? nullptr : w.rowub;
+        // each row's window bound starts its threshold
+        P.rowub = w.rowub;
+        P.ub_amax = pl.scaled ? amax : nullptr;
         P.ub_margin = kslack;
     }
     rc = launch_tiles(pl, w.G, w.rows_cap, w.ones, w.G, w.aug, w.rows_cap, P, grid, st, true);
@@ -3077,8 +2983,7 @@ size_t query_ws(int64_t N, int64_t nq, const KnnPlan& pl, QueryWs* out, void* ba
     w.na = cv.take<float>((size_t)w.capA + 512);
     w.nb = cv.take<float>((size_t)w.capB + 512);
     w.cand_id = pl.rerank ? cv.take<uint32_t>((size_t)nq * pl.kprime) : nullptr;
-    w.cand_d = pl.rerank ? cv.take<float>((size_t)nq * pl.kprime) : nullptr;
-    w.pool = cv.take<uint64_t>((size_t)w.capA * 2 * pool_half(pl.kprime));
+    w.pool = cv.take<uint64_t>((size_t)w.capA * 2 * pool_half(pl.kprime, pl.rerank));
     w.pool_cnt = cv.take<int>((size_t)w.capA * 2);
     w.srcA = cv.take<int64_t>((size_t)w.capA);
     w.srcB = cv.take<int64_t>((size_t)w.capB);
@@ -3133,7 +3038,7 @@ int run_knn_query(const void* X, int64_t N, const void* Q, int64_t nq, int d, in
     if (!rc) rc = launch_gather(X, dtype, d, w.srcB, w.capB, pl, w.GB, w.nb, w.augB, amax, st);
     if (rc) return rc;
     KnnParams P = base_params(pl, k, w.blk_off, w.prob, 1, w.na, nullptr, nullptr, 0, 0,
-                              pl.rerank ? w.cand_id : out_id, pl.rerank ? w.cand_d : out_d);
+                              pl.rerank ? w.cand_id : out_id, pl.rerank ? nullptr : out_d);
     P.pool = w.pool;
     P.pool_cnt = w.pool_cnt;
     const int64_t grid = (nq + kt::BM - 1) / kt::BM;

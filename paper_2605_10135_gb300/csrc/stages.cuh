@@ -102,8 +102,7 @@ struct KnnWs {
     __nv_bfloat16* ones;  // [128 x 16]: 1, 1, 1, then zeros
     float* norms;         // [rows_cap + 512]
     uint32_t* cand_id;  // [rows x kprime] when re-ranking
-    float* cand_d;
-    uint64_t* pool;     // [rows_cap x 2 x pool_half(kprime)] candidate pools of the sweeps
+    uint64_t* pool;     // [rows_cap x 2 x pool_half] candidate pools of the sweeps
     int* pool_cnt;      // [rows_cap x 2]
     int64_t rows_cap;
     // cell ordering
@@ -160,8 +159,7 @@ struct QueryWs {
     float* na;
     float* nb;
     uint32_t* cand_id;
-    float* cand_d;
-    uint64_t* pool;     // [capA x 2 x pool_half(kprime)] candidate pools of the sweep
+    uint64_t* pool;     // [capA x 2 x pool_half] candidate pools of the sweep
     int* pool_cnt;      // [capA x 2]
     int64_t capA, capB;
     int64_t* srcA;
