@@ -162,6 +162,10 @@ struct KnnParams {
     uint64_t* pool;
     int* pool_cnt;
     int ph;
+    // Column splits (queries): the problems are column ranges of one set of A rows, and
+    // the sorted list of pool row p goes to split_list[p k' ...] as (order bits of the
+    // key << 32 | id) instead of the outputs (NULL: no splits).
+    uint64_t* split_list;
     // Optional upper bound of every A row's k'-th squared distance (rowub[a]; NULL:
     // none): the sweep starts with that threshold.  Keys of split operands carry an
     // error, covered by the relative margin ub_margin (0 for exact keys); keys of
@@ -391,6 +395,7 @@ struct EpiState {
     volatile float* q_own;    // shared, this half's bounds of the warp's 32 rows
     volatile float* q_other;  // the other half's
     const uint32_t* gidrow;  // global id of each column of the shard (NULL: the column)
+    uint32_t id0;         // id of column 0 where gidrow is NULL
     uint32_t kscr;        // shared address of this thread's row of the warp's key scratch
     int kp, ph, c;
     float teff;
@@ -468,6 +473,33 @@ __device__ __forceinline__ void epi_compact(EpiState& s, uint32_t mask) {
     __syncwarp();
 }
 
+// The kp-th smallest of a thread's 32 keys (kp <= 32; NaN = +inf), by a sorting network
+// in registers (240 exchanges, one row per lane).
+template <int K, int J>
+__device__ __forceinline__ void sort32_from(float (&t)[32]) {  // stages (K, J) to (32, 1)
+#pragma unroll
+    for (int u = 0; u < 32; ++u)
+        if ((u ^ J) > u) {
+            const float a = fminf(t[u], t[u ^ J]), b = fmaxf(t[u], t[u ^ J]);
+            t[u] = (u & K) == 0 ? a : b;
+            t[u ^ J] = (u & K) == 0 ? b : a;
+        }
+    if constexpr (J > 1)
+        sort32_from<K, J / 2>(t);
+    else if constexpr (K < 32)
+        sort32_from<2 * K, K>(t);
+}
+__device__ __forceinline__ float kth_of_32(const float (&key)[32], int kp) {
+    float t[32];
+#pragma unroll
+    for (int u = 0; u < 32; ++u) t[u] = fminf(key[u], INFINITY);  // NaN -> +inf
+    sort32_from<2, 1>(t);
+    float b = t[31];
+#pragma unroll
+    for (int u = 0; u < 31; ++u) b = u == kp - 1 ? t[u] : b;
+    return b;
+}
+
 // One 32-column chunk: keys come straight from TMEM; masked columns become NaN
 // (every comparison with NaN is false, and the minimum skips NaN).  In a chunk with
 // survivors each thread marks its own, lays its keys out in the warp's scratch (8
@@ -505,7 +537,7 @@ __device__ __forceinline__ void epi_chunk(EpiState& s, const uint32_t (&v)[32], 
     if (PROF) ++s.c_slow;
     const int lane = threadIdx.x & 31;
     if (s.kp == 1) {  // the running minimum
-        uint32_t g_l = (uint32_t)(j0 + lane);  // global id of column j0 + lane
+        uint32_t g_l = s.id0 + (uint32_t)(j0 + lane);  // global id of column j0 + lane
         if (s.gidrow && j0 + lane < n_cols) g_l = __ldg(s.gidrow + j0 + lane);
 #pragma unroll
         for (int u = 0; u < 32; ++u) {
@@ -520,6 +552,17 @@ __device__ __forceinline__ void epi_chunk(EpiState& s, const uint32_t (&v)[32], 
         return;
     }
     s.teff = row_threshold(s.thr + lane);
+    // Short lists without a start threshold (queries, the centroid screen): the first
+    // chunk's k'-th key bounds the row's.  Without it every key of the first chunks
+    // goes to a pool of 64 entries, and each chunk is one compaction (about 5,000
+    // cycles) for each of the 32 rows.
+    if (s.kp <= 32 && __any_sync(0xffffffffu, s.teff == INFINITY)) {
+        const float b = kth_of_32(key, s.kp);
+        if (b < s.teff) {
+            atomicMin(s.thr + lane, f2ord(b));
+            s.teff = b;
+        }
+    }
     uint32_t surv = 0;  // bit u: column j0 + u survives for this row
 #pragma unroll
     for (int u = 0; u < 32; ++u) surv |= (key[u] <= s.teff ? 1u : 0u) << u;
@@ -594,7 +637,8 @@ __device__ __forceinline__ int tile_at(int tt, int t0, int ntiles) {
 }
 
 // EMX: pool entries per row half / 32 that the compaction holds in registers
-// (ph <= 32 EMX); the common pools (ph <= 256) use their own instantiation.
+// (ph <= 32 EMX); the common pools (ph <= 256) and the small ones (ph <= 96) use
+// instantiations of their own.
 template <int BN, bool PROF, int EMX>
 __global__ void __launch_bounds__(kt::THREADS, 1)
     k_knn_tiles(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUtensorMap tmB,
@@ -916,16 +960,16 @@ __global__ void __launch_bounds__(kt::THREADS, 1)
         EpiState s;
         const int i = rb * kt::BM + q * 32 + lane;  // row index inside the problem
         const int i0 = rb * kt::BM + q * 32;        // first row of this warp
-        const int64_t arow0 = pr.a_row0 + i0;       // gathered A row of lane 0
         s.ph = P.ph;
         s.c = 0;
         s.kp = P.kprime;
-        s.pool0 = P.pool + (arow0 * 2 + h) * (int64_t)P.ph;
+        s.pool0 = P.pool + ((pr.pool_row0 + i0) * 2 + h) * (int64_t)P.ph;
         s.thr = (uint32_t*)(base + L.tau) + q * 32;
         s.q_own = (volatile float*)(base + L.tau) + (1 + h) * kt::BM + q * 32;
         s.q_other = (volatile float*)(base + L.tau) + (2 - h) * kt::BM + q * 32;
         s.kscr = smem_u32(base + L.kscr) + ((warp - kt::EPI_WARP0) * 32 + lane) * 128;
         s.gidrow = P.gid ? P.gid + pr.b_row0 : nullptr;
+        s.id0 = pr.id0;
         s.best = ~0ull;
         s.teff = row_threshold(s.thr + lane);
         s.c_flush_cyc = s.c_chunks = s.c_slow = s.c_flushes = s.c_iters = s.c_app = 0;
@@ -1014,7 +1058,7 @@ __global__ void __launch_bounds__(kt::THREADS, 1)
             if (s.kp == 1)
                 s.pool0[(int64_t)lane * 2 * s.ph] = s.best;
             else
-                P.pool_cnt[(pr.a_row0 + i) * 2 + h] = ok ? s.c : 0;
+                P.pool_cnt[(pr.pool_row0 + i) * 2 + h] = ok ? s.c : 0;
         }
     }
     tc_fence_before();
@@ -1096,7 +1140,8 @@ __global__ void __launch_bounds__(1024)
         q.a_row0 = psh[sh];
         q.b_row0 = psh[sh];
         q.out_row0 = offsets[sh];
-        q.mem_row0 = offsets[sh];
+        q.pool_row0 = psh[sh];
+        q.id0 = 0;
         q.n_rows = (int32_t)ns;
         q.n_cols = (int32_t)ns;
         probs[s] = q;
@@ -1200,6 +1245,57 @@ __global__ void k_gather(const void* X, int dtype, int d, const int64_t* __restr
     }
 }
 
+// uint8 rows of d = 16 cd elements (16-byte aligned) into BF16 rows of Kp = 16 CP: CP lanes
+// a row (4, 8 or 16), 16 bytes in and two 16-byte stores out a lane.  Integer sums, so
+// the norms do not depend on the order.  k_gather's element loads and 2-byte stores
+// took 322 us for 1M rows of 128 (416 MB, floor 61 us); this takes 67 us.
+template <int CP>
+__global__ void __launch_bounds__(256)
+k_gather_u8(const uint8_t* __restrict__ X, int cd, const int64_t* __restrict__ srcrow,
+            int64_t rows_cap, __nv_bfloat16* __restrict__ G, float* __restrict__ norms,
+            __nv_bfloat16* __restrict__ aug) {
+    const int c = threadIdx.x % CP;
+    const int64_t step = (int64_t)gridDim.x * blockDim.x / CP;
+    // a warp's rows advance together, so every lane takes the same turns
+    const int64_t last = (rows_cap + 32 / CP - 1) / (32 / CP) * (32 / CP);
+    for (int64_t r = (blockIdx.x * (int64_t)blockDim.x + threadIdx.x) / CP; r < last; r += step) {
+        const int64_t src = r < rows_cap ? srcrow[r] : -1;
+        uint4 w = make_uint4(0, 0, 0, 0);
+        if (src >= 0 && c < cd) w = __ldg((const uint4*)X + src * cd + c);
+        const uint32_t in[4] = {w.x, w.y, w.z, w.w};
+        uint32_t o[8], n2 = 0;
+#pragma unroll
+        for (int q = 0; q < 4; ++q) {
+            n2 = __dp4a(in[q], in[q], n2);
+#pragma unroll
+            for (int b = 0; b < 2; ++b) {
+                const __nv_bfloat162 p = __floats2bfloat162_rn(
+                    (float)((in[q] >> (16 * b)) & 0xFFu), (float)((in[q] >> (16 * b + 8)) & 0xFFu));
+                o[2 * q + b] = *(const uint32_t*)&p;
+            }
+        }
+#pragma unroll
+        for (int m = CP / 2; m > 0; m >>= 1) n2 += __shfl_xor_sync(0xffffffffu, n2, m);
+        if (r >= rows_cap) continue;
+        uint4* g = (uint4*)G + (r * CP + c) * 2;
+        g[0] = make_uint4(o[0], o[1], o[2], o[3]);
+        g[1] = make_uint4(o[4], o[5], o[6], o[7]);
+        if (c == 0) {
+            const float nrm = (float)n2, half = 0.5f * nrm;
+            norms[r] = nrm;
+            const __nv_bfloat16 h = __float2bfloat16_rn(half);
+            const float r1 = half - __bfloat162float(h);
+            const __nv_bfloat16 m = __float2bfloat16_rn(r1);
+            const __nv_bfloat16 l = __float2bfloat16_rn(r1 - __bfloat162float(m));
+            const uint32_t hm = (uint32_t)__bfloat16_as_ushort(h) |
+                                ((uint32_t)__bfloat16_as_ushort(m) << 16);
+            uint4* a = (uint4*)(aug + r * kt::KAUG);
+            a[0] = make_uint4(hm, __bfloat16_as_ushort(l), 0, 0);
+            a[1] = make_uint4(0, 0, 0, 0);
+        }
+    }
+}
+
 // ---- row maps: which vector each gathered row holds ----------------------------
 __device__ __forceinline__ int shard_of_padded(const int64_t* __restrict__ pad_off, int C,
                                                int64_t pr) {
@@ -1260,7 +1356,8 @@ __global__ void k_pivot_tables(const int64_t* __restrict__ offsets, int C, int c
         pr.a_row0 = pad_off[s];
         pr.b_row0 = ppad_off[s];
         pr.out_row0 = offsets[s];
-        pr.mem_row0 = 0;
+        pr.pool_row0 = pad_off[s];
+        pr.id0 = 0;
         pr.n_rows = (int32_t)n;
         pr.n_cols = n > 0 ? npiv[s] : 0;
         pprobs[j] = pr;
@@ -1552,10 +1649,10 @@ k_pool_finalize(const KnnParams P) {
     for (int r = warp; r < kt::BM; r += 8) {
         const int i = rb * kt::BM + r;
         if (i >= pr.n_rows) break;
-        const int64_t arow = pr.a_row0 + i;
-        const int c0 = min(max(P.pool_cnt[arow * 2], 0), P.ph);
-        const int c1 = min(max(P.pool_cnt[arow * 2 + 1], 0), P.ph);
-        const uint64_t* h0 = P.pool + arow * 2 * (int64_t)P.ph;
+        const int64_t prow = pr.pool_row0 + i;
+        const int c0 = min(max(P.pool_cnt[prow * 2], 0), P.ph);
+        const int c1 = min(max(P.pool_cnt[prow * 2 + 1], 0), P.ph);
+        const uint64_t* h0 = P.pool + prow * 2 * (int64_t)P.ph;
         const uint64_t* h1 = h0 + P.ph;
         uint64_t v[2 * EH];
 #pragma unroll
@@ -1587,10 +1684,18 @@ k_pool_finalize(const KnnParams P) {
         for (int e = 0; e < KE; ++e) {
             w[e] = stg[lane * KE + e];
             if (w[e] != ~0ull)
-                w[e] = (w[e] & 0xFFFFFFFF00000000ull) | column_gid(gidrow, (uint32_t)w[e]);
+                w[e] = (w[e] & 0xFFFFFFFF00000000ull) |
+                       (pr.id0 + column_gid(gidrow, (uint32_t)w[e]));
         }
         __syncwarp();
         warp_bitonic_u64<KE>(w);
+        if (P.split_list) {
+#pragma unroll
+            for (int e = 0; e < KE; ++e)
+                if (lane * KE + e < kp) P.split_list[prow * kp + lane * KE + e] = w[e];
+            continue;
+        }
+        const int64_t arow = pr.a_row0 + i;
         const float nx = P.na[arow];
         const int64_t orow = P.outrow ? P.outrow[arow] : pr.out_row0 + i;
 #pragma unroll
@@ -1623,11 +1728,15 @@ __global__ void __launch_bounds__(kt::BM) k_pool_finalize1(const KnnParams P) {
     const KnnProblem pr = P.probs[lo];
     const int i = (int)(bid - P.blk_off[lo]) * kt::BM + (int)threadIdx.x;
     if (i >= pr.n_rows) return;
-    const int64_t arow = pr.a_row0 + i;
-    const uint64_t* h0 = P.pool + arow * 2 * (int64_t)P.ph;
+    const int64_t arow = pr.a_row0 + i, prow = pr.pool_row0 + i;
+    const uint64_t* h0 = P.pool + prow * 2 * (int64_t)P.ph;
     const uint64_t a = h0[0];
     const uint64_t b = h0[P.ph];
     const uint64_t w = a < b ? a : b;
+    if (P.split_list) {
+        P.split_list[prow] = w;
+        return;
+    }
     const int64_t orow = P.outrow ? P.outrow[arow] : pr.out_row0 + i;
     uint32_t id = ANN_PAD;
     float dd = INFINITY;
@@ -1636,10 +1745,43 @@ __global__ void __launch_bounds__(kt::BM) k_pool_finalize1(const KnnParams P) {
         dd = fmaf(2.0f, ord2f((uint32_t)(w >> 32)), P.na[arow]);
     }
     P.out_id[orow * P.k_out] = id;
-    P.out_d[orow * P.k_out] = dd;
+    if (P.out_d) P.out_d[orow * P.k_out] = dd;
     for (int slot = 1; slot < P.k_out; ++slot) {
         P.out_id[orow * P.k_out + slot] = ANN_PAD;
-        P.out_d[orow * P.k_out + slot] = INFINITY;
+        if (P.out_d) P.out_d[orow * P.k_out + slot] = INFINITY;
+    }
+}
+
+// Column splits: row i's sorted lists of the ns <= 32 splits (split s at pool row
+// s stride + i) merged into its first k_out entries.  One warp per row, lane = split:
+// each turn takes the smallest head (key, id).  k_out turns of two warp minima and one
+// L2 access by the winning lane, on lists of 26 entries some 20 us for all rows.
+__global__ void __launch_bounds__(128)
+k_split_merge(const uint64_t* __restrict__ lists, int ns, int64_t stride, int kp, int64_t nrows,
+              int k_out, const float* __restrict__ na, uint32_t* __restrict__ out_id,
+              float* __restrict__ out_d) {
+    const int lane = threadIdx.x & 31;
+    const int64_t i = (blockIdx.x * (int64_t)blockDim.x + threadIdx.x) >> 5;
+    if (i >= nrows) return;
+    const uint64_t* mine = lists + ((int64_t)lane * stride + i) * kp;
+    uint64_t cur = lane < ns ? mine[0] : ~0ull;
+    uint64_t nxt = lane < ns && kp > 1 ? mine[1] : ~0ull;
+    int at = 2;
+    const float nx = na[i];
+    for (int o = 0; o < k_out; ++o) {
+        const uint32_t hi = __reduce_min_sync(0xffffffffu, (uint32_t)(cur >> 32));
+        const bool tied = (uint32_t)(cur >> 32) == hi;
+        const uint32_t id = __reduce_min_sync(0xffffffffu, tied ? (uint32_t)cur : 0xFFFFFFFFu);
+        const bool pad = hi == 0xFFFFFFFFu;
+        if (lane == 0) {
+            out_id[i * k_out + o] = pad ? ANN_PAD : id;
+            if (out_d) out_d[i * k_out + o] = pad ? INFINITY : fmaf(2.0f, ord2f(hi), nx);
+        }
+        if (!pad && tied && (uint32_t)cur == id) {  // one lane: the splits' ids are disjoint
+            cur = nxt;
+            nxt = at < kp ? mine[at] : ~0ull;
+            ++at;
+        }
     }
 }
 
@@ -2575,12 +2717,16 @@ static int launch_tiles(const KnnPlan& pl, const void* GA, int64_t rowsA, const 
     if (rc) return rc;
     const bool prof = timed && tile_counters_on();
     constexpr int EBIG = kt::PH_MAX / 32;
-    const bool big = P.ph > 256;
+    const bool big = P.ph > 256, small = P.ph <= 96;
     auto kern = pl.bn == 256
                     ? (prof ? k_knn_tiles<256, true, EBIG>
-                            : big ? k_knn_tiles<256, false, EBIG> : k_knn_tiles<256, false, 8>)
+                            : big   ? k_knn_tiles<256, false, EBIG>
+                            : small ? k_knn_tiles<256, false, 3>
+                                    : k_knn_tiles<256, false, 8>)
                     : (prof ? k_knn_tiles<128, true, EBIG>
-                            : big ? k_knn_tiles<128, false, EBIG> : k_knn_tiles<128, false, 8>);
+                            : big   ? k_knn_tiles<128, false, EBIG>
+                            : small ? k_knn_tiles<128, false, 3>
+                                    : k_knn_tiles<128, false, 8>);
     ANN_CHECK_CUDA(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                         (int)pl.smem));
     if (grid <= 0) return ANN_OK;
@@ -2721,6 +2867,7 @@ static KnnParams base_params(const KnnPlan& pl, int k, const int64_t* blk_off,
     P.rowub = nullptr;
     P.ub_margin = 0.0f;
     P.ub_amax = nullptr;
+    P.split_list = nullptr;
     return P;
 }
 
@@ -2730,6 +2877,17 @@ static int launch_gather(const void* X, int dtype, int d, const int64_t* src, in
     const int threads = 256;
     const int64_t want = (rows_cap * 32 + threads - 1) / threads;
     const unsigned grid = (unsigned)(want < 152 * 64 ? want : 152 * 64);
+    const int cp = pl.Kp / 16;
+    if (dtype == ANN_U8 && pl.mode == 0 && !pl.elem8 && pl.ab_fmt == 1 && !pl.scaled &&
+        d % 16 == 0 && ((uintptr_t)X & 15) == 0 && (cp == 4 || cp == 8 || cp == 16)) {
+        const int64_t blocks = (rows_cap * cp + 255) / 256;
+        const unsigned g = (unsigned)(blocks < 152 * 32 ? blocks : 152 * 32);
+        const auto kern = cp == 4 ? k_gather_u8<4> : cp == 8 ? k_gather_u8<8> : k_gather_u8<16>;
+        kern<<<g, 256, 0, st>>>((const uint8_t*)X, d / 16, src, rows_cap, (__nv_bfloat16*)G, norms,
+                                aug);
+        ANN_CHECK_LAUNCH();
+        return ANN_OK;
+    }
     if (pl.elem8)
         k_gather<__nv_fp8_e4m3><<<grid, threads, 0, st>>>(X, dtype, d, src, rows_cap, pl.mode,
                                                           pl.Kp, pl.Kh, (__nv_fp8_e4m3*)G, norms,
@@ -2965,16 +3123,38 @@ int run_shard_knn(const void* X, int64_t N, int d, int dtype, const uint32_t* me
     return ANN_OK;
 }
 
-// Query side: A = queries, B = all N vectors (one problem, no self exclusion).
+// Query side: A = queries, B = all N vectors (no self exclusion).  With fewer row blocks
+// than SMs the columns are split into ns ranges of whole tiles, each a problem of its
+// own with pools of its own, and k_split_merge merges their sorted lists.  ns (at most
+// 32, one lane each in the merge) minimises waves x (tiles a range + 6): a range starts
+// without thresholds, which costs it about six tiles.  1,000 queries over 1M uint8
+// vectors (8 row blocks): 8 CTAs of 3,907 tiles took 5.6 ms, 152 of 206 take 0.74 ms
+// (a range meets more survivors than the whole: k' (1 + ln(n / k')) a range).
+constexpr int QS_MAX = 32;
+static int query_splits(int64_t N, int64_t nq) {
+    const int64_t nb = (nq + kt::BM - 1) / kt::BM, tiles = (N + kt::BNMAX - 1) / kt::BNMAX;
+    int best = 1;
+    double cost = 0.0;
+    for (int ns = 1; ns <= QS_MAX && ns <= tiles && (ns == 1 || nb * ns <= 2 * 152); ++ns) {
+        const int64_t per = (tiles + ns - 1) / ns;
+        const double c = (double)((nb * ns + 151) / 152) * (double)(per + 6);
+        if (ns == 1 || c < cost) {
+            best = ns;
+            cost = c;
+        }
+    }
+    return best;
+}
 size_t query_ws(int64_t N, int64_t nq, const KnnPlan& pl, QueryWs* out, void* base, size_t cap) {
     Carver cv(base, cap);
     QueryWs w;
     w.capA = nq + kt::BM + kt::BNMAX;
     w.capB = N + kt::BM + kt::BNMAX;
-    w.blk_off = cv.take<int64_t>(4);
+    w.blk_off = cv.take<int64_t>(QS_MAX + 1);
     w.pad_off = cv.take<int64_t>(4);
     w.offs = cv.take<int64_t>(4);
-    w.prob = cv.take<KnnProblem>(1);
+    const int ns = query_splits(N, nq);
+    w.prob = cv.take<KnnProblem>(QS_MAX);
     w.GA = (__nv_bfloat16*)cv.take<uint8_t>((size_t)w.capA * row_bytes(pl));
     w.GB = (__nv_bfloat16*)cv.take<uint8_t>((size_t)w.capB * row_bytes(pl));
     w.augA = cv.take<__nv_bfloat16>((size_t)w.capA * kt::KAUG);
@@ -2983,8 +3163,12 @@ size_t query_ws(int64_t N, int64_t nq, const KnnPlan& pl, QueryWs* out, void* ba
     w.na = cv.take<float>((size_t)w.capA + 512);
     w.nb = cv.take<float>((size_t)w.capB + 512);
     w.cand_id = pl.rerank ? cv.take<uint32_t>((size_t)nq * pl.kprime) : nullptr;
-    w.pool = cv.take<uint64_t>((size_t)w.capA * 2 * pool_half(pl.kprime, pl.rerank));
-    w.pool_cnt = cv.take<int>((size_t)w.capA * 2);
+    w.ns = ns;
+    w.pstride = ns > 1 ? (nq + kt::BM - 1) / kt::BM * kt::BM : 0;
+    const int64_t prows = ns > 1 ? ns * w.pstride : w.capA;
+    w.pool = cv.take<uint64_t>((size_t)prows * 2 * pool_half(pl.kprime, pl.rerank));
+    w.pool_cnt = cv.take<int>((size_t)prows * 2);
+    w.split_list = ns > 1 ? cv.take<uint64_t>((size_t)prows * pl.kprime) : nullptr;
     w.srcA = cv.take<int64_t>((size_t)w.capA);
     w.srcB = cv.take<int64_t>((size_t)w.capB);
     w.amax = cv.take<float>(4);
@@ -2992,33 +3176,56 @@ size_t query_ws(int64_t N, int64_t nq, const KnnPlan& pl, QueryWs* out, void* ba
     return cv.used + 256;
 }
 
-__global__ void k_query_tables(int64_t N, int64_t nq, int64_t* blk_off, int64_t* pad4,
-                               int64_t* offs4, KnnProblem* prob) {
+__global__ void k_query_tables(int64_t N, int64_t nq, int ns, int64_t pstride, int64_t* blk_off,
+                               int64_t* pad4, int64_t* offs4, KnnProblem* prob) {
     if (threadIdx.x || blockIdx.x) return;
-    blk_off[0] = 0;
-    blk_off[1] = (nq + kt::BM - 1) / kt::BM;
+    const int64_t nb = (nq + kt::BM - 1) / kt::BM;
     offs4[0] = 0;  // A side (queries): offsets {0, nq}, padded {0, nq rounded up}
     offs4[1] = nq;
     offs4[2] = 0;  // B side (all vectors): offsets {0, N}
     offs4[3] = N;
     pad4[0] = 0;
-    pad4[1] = blk_off[1] * kt::BM;
+    pad4[1] = nb * kt::BM;
     pad4[2] = 0;
     pad4[3] = (N + kt::BM - 1) / kt::BM * kt::BM;
-    KnnProblem p;
-    p.a_row0 = 0;
-    p.b_row0 = 0;
-    p.out_row0 = 0;
-    p.mem_row0 = 0;
-    p.n_rows = (int32_t)nq;
-    p.n_cols = (int32_t)N;
-    prob[0] = p;
+    const int64_t tiles = (N + kt::BNMAX - 1) / kt::BNMAX;
+    const int64_t cols = (tiles + ns - 1) / ns * kt::BNMAX;
+    for (int s = 0; s < ns; ++s) {
+        const int64_t c0 = s * cols < N ? s * cols : N;
+        KnnProblem p;
+        p.a_row0 = 0;
+        p.b_row0 = c0;
+        p.out_row0 = 0;
+        p.pool_row0 = s * pstride;
+        p.id0 = (uint32_t)c0;
+        p.n_rows = (int32_t)nq;
+        p.n_cols = (int32_t)(N - c0 < cols ? N - c0 : cols);
+        prob[s] = p;
+        blk_off[s] = s * nb;
+    }
+    blk_off[ns] = ns * nb;
+}
+
+// The tile launch over a query's splits and, with more than one, the merge.
+static int query_sweep(const KnnPlan& pl, const QueryWs& w, int64_t nq, KnnParams P,
+                       cudaStream_t st, bool timed) {
+    P.pool = w.pool;
+    P.pool_cnt = w.pool_cnt;
+    P.split_list = w.split_list;
+    const int64_t grid = w.ns * ((nq + kt::BM - 1) / kt::BM);
+    int rc = launch_tiles(pl, w.GA, w.capA, w.ones, w.GB, w.augB, w.capB, P, grid, st, timed);
+    if (rc || w.ns == 1 || grid == 0) return rc;
+    k_split_merge<<<(unsigned)((nq + 3) / 4), 128, 0, st>>>(w.split_list, w.ns, w.pstride,
+                                                            P.kprime, nq, P.k_out, P.na, P.out_id,
+                                                            P.out_d);
+    ANN_CHECK_LAUNCH();
+    return ANN_OK;
 }
 
 int run_knn_query(const void* X, int64_t N, const void* Q, int64_t nq, int d, int dtype, int k,
                   const KnnPlan& pl, const QueryWs& w, uint32_t* out_id, float* out_d,
                   cudaStream_t st) {
-    k_query_tables<<<1, 32, 0, st>>>(N, nq, w.blk_off, w.pad_off, w.offs, w.prob);
+    k_query_tables<<<1, 32, 0, st>>>(N, nq, w.ns, w.pstride, w.blk_off, w.pad_off, w.offs, w.prob);
     ANN_CHECK_LAUNCH();
     k_ones_tile<<<(128 * kt::KAUG + 255) / 256, 256, 0, st>>>(w.ones);
     ANN_CHECK_LAUNCH();
@@ -3037,12 +3244,9 @@ int run_knn_query(const void* X, int64_t N, const void* Q, int64_t nq, int d, in
     int rc = launch_gather(Q, dtype, d, w.srcA, w.capA, pl, w.GA, w.na, w.augA, amax, st);
     if (!rc) rc = launch_gather(X, dtype, d, w.srcB, w.capB, pl, w.GB, w.nb, w.augB, amax, st);
     if (rc) return rc;
-    KnnParams P = base_params(pl, k, w.blk_off, w.prob, 1, w.na, nullptr, nullptr, 0, 0,
-                              pl.rerank ? w.cand_id : out_id, pl.rerank ? nullptr : out_d);
-    P.pool = w.pool;
-    P.pool_cnt = w.pool_cnt;
-    const int64_t grid = (nq + kt::BM - 1) / kt::BM;
-    rc = launch_tiles(pl, w.GA, w.capA, w.ones, w.GB, w.augB, w.capB, P, grid, st, true);
+    const KnnParams P = base_params(pl, k, w.blk_off, w.prob, w.ns, w.na, nullptr, nullptr, 0, 0,
+                                    pl.rerank ? w.cand_id : out_id, pl.rerank ? nullptr : out_d);
+    rc = query_sweep(pl, w, nq, P, st, true);
     if (rc) return rc;
     if (pl.rerank)
         return launch_rerank(X, Q, dtype, d, nullptr, nq, w.cand_id, pl.kprime, k, out_id, out_d,
@@ -3107,7 +3311,7 @@ int run_screen(const void* Xa, int dta, const uint32_t* rowsel, int64_t p0, int6
     float* out_d = cv.take<float>((size_t)na * ks);
     QueryWs w;
     query_ws(nb, na, pl, &w, qbase, qb);
-    k_query_tables<<<1, 32, 0, st>>>(nb, na, w.blk_off, w.pad_off, w.offs, w.prob);
+    k_query_tables<<<1, 32, 0, st>>>(nb, na, w.ns, w.pstride, w.blk_off, w.pad_off, w.offs, w.prob);
     ANN_CHECK_LAUNCH();
     k_ones_tile<<<(128 * kt::KAUG + 255) / 256, 256, 0, st>>>(w.ones);
     ANN_CHECK_LAUNCH();
@@ -3120,12 +3324,9 @@ int run_screen(const void* Xa, int dta, const uint32_t* rowsel, int64_t p0, int6
         return rc;
     if ((rc = launch_gather(Xb, dtb, d, w.srcB, w.capB, pl, w.GB, w.nb, w.augB, nullptr, st)))
         return rc;
-    KnnParams P = base_params(pl, ks, w.blk_off, w.prob, 1, w.na, nullptr, nullptr, 0, 0, out_id,
-                              out_d);
-    P.pool = w.pool;
-    P.pool_cnt = w.pool_cnt;
-    const int64_t grid = (na + kt::BM - 1) / kt::BM;
-    return launch_tiles(pl, w.GA, w.capA, w.ones, w.GB, w.augB, w.capB, P, grid, st, false);
+    const KnnParams P = base_params(pl, ks, w.blk_off, w.prob, w.ns, w.na, nullptr, nullptr, 0, 0,
+                                    out_id, out_d);
+    return query_sweep(pl, w, na, P, st, false);
 }
 
 }  // namespace ann

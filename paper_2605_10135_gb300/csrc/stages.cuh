@@ -66,7 +66,8 @@ struct KnnProblem {
     int64_t a_row0;    // first row of the problem in the A buffer (padded index space)
     int64_t b_row0;    // first row in the B buffer
     int64_t out_row0;  // first output row
-    int64_t mem_row0;  // members[] offset of column 0 (global id lookup)
+    int64_t pool_row0; // first row of its candidate pools
+    uint32_t id0;      // id of column 0 where no id table is given
     int32_t n_rows, n_cols;
 };
 
@@ -159,8 +160,11 @@ struct QueryWs {
     float* na;
     float* nb;
     uint32_t* cand_id;
-    uint64_t* pool;     // [capA x 2 x pool_half] candidate pools of the sweep
-    int* pool_cnt;      // [capA x 2]
+    int ns;             // column splits
+    int64_t pstride;    // pool rows of one split (ns > 1)
+    uint64_t* pool;     // [rows x 2 x pool_half] candidate pools of the sweep
+    int* pool_cnt;      // [rows x 2], rows = ns pstride (capA without splits)
+    uint64_t* split_list;  // [rows x kprime] sorted lists of the splits (ns > 1)
     int64_t capA, capB;
     int64_t* srcA;
     int64_t* srcB;
