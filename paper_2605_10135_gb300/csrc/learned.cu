@@ -46,11 +46,14 @@ __device__ __forceinline__ float mat_at(const Mat& m, int64_t r, int64_t c, floa
     return load_elem(m.p, m.dtype, row * m.ld + sc) * s;
 }
 
-// C[M x N] = A[M x K] . B[K x N], ep(i, j, acc) stores each output.
+// C[M x N] = A[M x K] . B[K x N], ep(i, j, acc) stores each output.  K goes through
+// shared memory 64 at a time: the products of a training step have K = 32 or slices of
+// 64, so all their loads are in flight at once (16 at a time made four round trips).
+constexpr int SK = 64;
 template <class EP>
 __global__ void __launch_bounds__(256) k_sgemm(int64_t M, int N, int K, Mat A, Mat B, EP ep) {
-    __shared__ float As[16][68];
-    __shared__ float Bs[16][68];
+    __shared__ float As[SK][68];
+    __shared__ float Bs[SK][68];
     const int t = threadIdx.x, tx = t & 15, ty = t >> 4;
     const int64_t m0 = (int64_t)blockIdx.x * 64;
     const int n0 = blockIdx.y * 64;
@@ -60,27 +63,28 @@ __global__ void __launch_bounds__(256) k_sgemm(int64_t M, int N, int K, Mat A, M
     for (int i = 0; i < 4; ++i)
 #pragma unroll
         for (int j = 0; j < 4; ++j) acc[i][j] = 0.0f;
-    for (int k0 = 0; k0 < K; k0 += 16) {
+    for (int k0 = 0; k0 < K; k0 += SK) {
 #pragma unroll
-        for (int q = 0; q < 4; ++q) {
+        for (int q = 0; q < SK / 4; ++q) {
             const int e = t + q * 256;
-            const int r = A.trans ? (e & 63) : (e >> 4);  // consecutive threads follow
-            const int c = A.trans ? (e >> 6) : (e & 15);  // the stored rows
+            const int r = A.trans ? (e & 63) : (e / SK);  // consecutive threads follow
+            const int c = A.trans ? (e >> 6) : (e % SK);  // the stored rows
             const int64_t gi = m0 + r;
             const int gk = k0 + c;
             As[c][r] = (gi < M && gk < K) ? mat_at(A, gi, gk, sa) : 0.0f;
         }
 #pragma unroll
-        for (int q = 0; q < 4; ++q) {
+        for (int q = 0; q < SK / 4; ++q) {
             const int e = t + q * 256;
-            const int r = B.trans ? (e & 15) : (e >> 6);
-            const int c = B.trans ? (e >> 4) : (e & 63);
+            const int r = B.trans ? (e % SK) : (e >> 6);
+            const int c = B.trans ? (e / SK) : (e & 63);
             const int gk = k0 + r, gj = n0 + c;
             Bs[r][c] = (gk < K && gj < N) ? mat_at(B, gk, gj, sb) : 0.0f;
         }
         __syncthreads();
-#pragma unroll
-        for (int kk = 0; kk < 16; ++kk) {
+        const int ke = K - k0 < SK ? K - k0 : SK;
+#pragma unroll 8
+        for (int kk = 0; kk < ke; ++kk) {
             float a[4], b[4];
 #pragma unroll
             for (int i = 0; i < 4; ++i) a[i] = As[kk][ty * 4 + i];
@@ -164,8 +168,8 @@ __global__ void __launch_bounds__(256)
     }
     EpPart ep{part + (int64_t)z * M * N, M, N};
     // same tile loop as k_sgemm on the slice
-    __shared__ float As[16][68];
-    __shared__ float Bs[16][68];
+    __shared__ float As[SK][68];
+    __shared__ float Bs[SK][68];
     const int t = threadIdx.x, tx = t & 15, ty = t >> 4;
     const int64_t m0 = (int64_t)blockIdx.x * 64;
     const int n0 = blockIdx.y * 64;
@@ -175,27 +179,28 @@ __global__ void __launch_bounds__(256)
     for (int i = 0; i < 4; ++i)
 #pragma unroll
         for (int j = 0; j < 4; ++j) acc[i][j] = 0.0f;
-    for (int kk0 = 0; kk0 < kn; kk0 += 16) {
+    for (int kk0 = 0; kk0 < kn; kk0 += SK) {
 #pragma unroll
-        for (int q = 0; q < 4; ++q) {
+        for (int q = 0; q < SK / 4; ++q) {
             const int e = t + q * 256;
-            const int r = a.trans ? (e & 63) : (e >> 4);
-            const int c = a.trans ? (e >> 6) : (e & 15);
+            const int r = a.trans ? (e & 63) : (e / SK);
+            const int c = a.trans ? (e >> 6) : (e % SK);
             const int64_t gi = m0 + r;
             const int gk = kk0 + c;
             As[c][r] = (gi < M && gk < kn) ? mat_at(a, gi, gk, sa) : 0.0f;
         }
 #pragma unroll
-        for (int q = 0; q < 4; ++q) {
+        for (int q = 0; q < SK / 4; ++q) {
             const int e = t + q * 256;
-            const int r = b.trans ? (e & 15) : (e >> 6);
-            const int c = b.trans ? (e >> 4) : (e & 63);
+            const int r = b.trans ? (e % SK) : (e >> 6);
+            const int c = b.trans ? (e / SK) : (e & 63);
             const int gk = kk0 + r, gj = n0 + c;
             Bs[r][c] = (gk < kn && gj < N) ? mat_at(b, gk, gj, sb) : 0.0f;
         }
         __syncthreads();
-#pragma unroll
-        for (int kk = 0; kk < 16; ++kk) {
+        const int ke = kn - kk0 < SK ? kn - kk0 : SK;
+#pragma unroll 8
+        for (int kk = 0; kk < ke; ++kk) {
             float av[4], bv[4];
 #pragma unroll
             for (int i = 0; i < 4; ++i) av[i] = As[kk][ty * 4 + i];
@@ -276,12 +281,16 @@ static Mat mat(const void* p, int dtype, int64_t ld, int trans = 0, const uint32
 // ---- tensor-core GEMM of the training step ------------------------------------
 // D[M x N] (FP32) = A[M x K] . B[N x K]^T, BF16 operands stored K-major with rows
 // padded to whole tiles (missing rows of the tensor map read as zeros) and K a
-// multiple of 64.  One 128 x 256 output tile per CTA, the K blocks of slice
-// blockIdx.z: warp 0 issues TMA copies into a ring of 3 stages, warp 1 the
-// tcgen05.mma (FP32 accumulator in TMEM), then every warp reads its 32 rows
-// back (thread = row) and hands ep(row, col, value, slice) each output.
+// multiple of 64.  One 128 x 64 output tile per CTA, the K blocks of slice
+// blockIdx.z: warp 0 issues TMA copies into a ring of 8 stages, one elected lane of
+// warp 1 the tcgen05.mma (FP32 accumulator in TMEM), then every warp reads its 32 rows
+// back (thread = row) and hands ep(row, col, value, slice) each output.  A training
+// step's products are small (1,536 x 256 outputs, K = 3 d): what counts is CTAs and
+// bytes in flight, since each CTA walks all K blocks of its slice in turn and the sums
+// over K keep their order.  128 x 256 tiles with 3 stages left 12 CTAs: 74 us at
+// d = 1024, now 28 (the weight gradient 27 us, now 20).
 namespace tgm {
-constexpr int BM = 128, BN = 256, KB = 64, NST = 3;
+constexpr int BM = 128, BN = 64, KB = 64, NST = 8;
 constexpr int A_BYTES = BM * 128, B_BYTES = BN * 128, STAGE = A_BYTES + B_BYTES;
 constexpr int THREADS = 128;
 constexpr size_t SMEM = 1024 + (size_t)NST * STAGE + (2 * NST + 1) * 8 + 16;
@@ -300,7 +309,8 @@ __global__ void __launch_bounds__(tgm::THREADS, 1)
     const uint32_t full = bars, empty = bars + NST * 8, done = bars + 2 * NST * 8;
     volatile uint32_t* tslot = (volatile uint32_t*)(tail + (2 * NST + 1) * 8);
     volatile int* abort_flag = (volatile int*)(tslot + 1);
-    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const int warp = __shfl_sync(0xffffffffu, (int)(threadIdx.x >> 5), 0);
+    const int lane = threadIdx.x & 31;
     const int64_t m0 = (int64_t)blockIdx.x * BM;
     const int n0 = blockIdx.y * BN;
     const int kb0 = blockIdx.z * kb_per_slice;
@@ -341,21 +351,25 @@ __global__ void __launch_bounds__(tgm::THREADS, 1)
         for (int st = 0; st < NST; ++st)
             if (used >> st & 1) mbar_wait(full + 8 * st, (last_par >> st) & 1u, &dummy, 200000000ull);
         if (!ok) atomicOr(status, DEV_TIMEOUT);
-    } else if (warp == 1 && lane == 0) {
+    } else if (warp == 1) {
         for (int kb = kb0; kb < kb1; ++kb) {
             const int i = kb - kb0, st = i % NST;
             const uint32_t ph = (uint32_t)(i / NST) & 1u;
-            if (!mbar_wait(full + 8 * st, ph, abort_flag)) { ok = false; break; }
+            ok = mbar_wait_warp(full + 8 * st, ph, abort_flag);
+            if (!ok) break;
             tc_fence_after();
             const uint32_t a = ring + st * STAGE, b = a + A_BYTES;
+            if (elect_one()) {
 #pragma unroll
-            for (int q = 0; q < 4; ++q)
-                umma_f16(tmem, sdesc_sw128(a + q * 32), sdesc_sw128(b + q * 32), idesc,
-                         (i | q) != 0 ? 1u : 0u);
-            umma_commit(empty + 8 * st);
+                for (int q = 0; q < 4; ++q)
+                    umma_f16(tmem, sdesc_sw128(a + q * 32), sdesc_sw128(b + q * 32), idesc,
+                             (i | q) != 0 ? 1u : 0u);
+                umma_commit(empty + 8 * st);
+            }
+            __syncwarp();
         }
-        umma_commit(done);  // also after a timeout: every issued MMA completes first
-        if (!ok) atomicOr(status, DEV_TIMEOUT);
+        if (elect_one()) umma_commit(done);  // also after a timeout: every issued MMA completes first
+        if (!ok && lane == 0) atomicOr(status, DEV_TIMEOUT);
     }
     __syncwarp();
     const bool got = mbar_wait(done, 0, abort_flag);
@@ -416,15 +430,22 @@ __device__ __forceinline__ void bf16_split(float v, __nv_bfloat16& hi, __nv_bflo
     hi = __float2bfloat16_rn(v);
     lo = __float2bfloat16_rn(v - __bfloat162float(hi));
 }
-__global__ void k_batch_bf16(const void* X, int dtype, int d, const uint32_t* __restrict__ idx,
-                             int64_t R, int64_t Rp, int Kp, const float* __restrict__ inv_s,
-                             __nv_bfloat16* __restrict__ rows, __nv_bfloat16* __restrict__ cols) {
+// One 32 x 32 tile per block turn, transposed through shared memory so that both forms
+// are written in runs of 64 bytes (element-wise transposed stores took 44 us for 1,536
+// rows of 1,024, this BA28).
+__global__ void __launch_bounds__(256)
+k_batch_bf16(const void* X, int dtype, int d, const uint32_t* __restrict__ idx, int64_t R,
+             int64_t Rp, int Kp, const float* __restrict__ inv_s, __nv_bfloat16* __restrict__ rows,
+             __nv_bfloat16* __restrict__ cols) {
+    __shared__ __nv_bfloat16 th[32][34], tl[32][34];
     const float sc = *inv_s;
-    const int64_t tot = Rp * Kp;
-    for (int64_t q = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; q < tot;
-         q += (int64_t)gridDim.x * blockDim.x) {
-        const int64_t r = q / Kp;
-        const int t = (int)(q - r * Kp);
+    const int tx = threadIdx.x & 31, ty = threadIdx.x >> 5;  // Rp and Kp are multiples of 32
+    const int64_t r0 = (int64_t)blockIdx.y * 32;
+    const int t0 = blockIdx.x * 32;
+#pragma unroll
+    for (int q = 0; q < 4; ++q) {
+        const int64_t r = r0 + ty + 8 * q;
+        const int t = t0 + tx;
         const float v = (r < R && t < d) ? load_elem(X, dtype, (int64_t)idx[r] * d + t) * sc : 0.0f;
         __nv_bfloat16 hi, lo;
         bf16_split(v, hi, lo);
@@ -432,7 +453,14 @@ __global__ void k_batch_bf16(const void* X, int dtype, int d, const uint32_t* __
         rw[0] = hi;
         rw[Kp] = lo;
         rw[2 * Kp] = hi;
-        __nv_bfloat16* cl = cols + (int64_t)t * 3 * Rp + r;
+        th[ty + 8 * q][tx] = hi;
+        tl[ty + 8 * q][tx] = lo;
+    }
+    __syncthreads();
+#pragma unroll
+    for (int q = 0; q < 4; ++q) {
+        const __nv_bfloat16 hi = th[tx][ty + 8 * q], lo = tl[tx][ty + 8 * q];
+        __nv_bfloat16* cl = cols + (int64_t)(t0 + ty + 8 * q) * 3 * Rp + r0 + tx;
         cl[0] = hi;
         cl[Rp] = hi;
         cl[2 * Rp] = lo;
@@ -511,7 +539,19 @@ __device__ __forceinline__ uint32_t safe_id(uint32_t v, int64_t N, int* status) 
 __global__ void k_triplets(const uint32_t* __restrict__ sample, int64_t S,
                            const uint32_t* __restrict__ knn, int kk, int kpos,
                            const uint32_t* __restrict__ draws, const int* __restrict__ step,
-                           int B, int64_t N, uint32_t* __restrict__ idx, int* status) {
+                           int B, int64_t N, uint32_t* __restrict__ idx, float* __restrict__ coef,
+                           int* status) {
+    if (blockIdx.x == gridDim.x - 1) {
+        // Adam's bias corrections of this step (t = *step + 1), in double and rounded
+        // once: one thread in a block of its own (a pair of pow() per parameter took
+        // 91 us a step at d = 1024)
+        if (threadIdx.x == 0) {
+            const double t = (double)(*step + 1);
+            coef[0] = (float)(1.0 / (1.0 - pow(0.9, t)));
+            coef[1] = (float)(1.0 / (1.0 - pow(0.999, t)));
+        }
+        return;
+    }
     const int i = blockIdx.x * blockDim.x + threadIdx.x;
     if (i >= B) return;
     const uint32_t* dr = draws + ((int64_t)*step * B + i) * 3;
@@ -533,9 +573,18 @@ __global__ void k_triplet_loss(const float* __restrict__ Z, int B, float margin,
     const float* za = Z + (int64_t)i * ml::OUT;
     const float* zp = Z + (int64_t)(B + i) * ml::OUT;
     const float* zn = Z + (int64_t)(2 * B + i) * ml::OUT;
+    // the three rows first (24 independent 16-byte loads), then the sums in order
+    float a[ml::OUT], pz[ml::OUT], nz[ml::OUT];
+#pragma unroll
+    for (int c = 0; c < ml::OUT / 4; ++c) {
+        *(float4*)(a + 4 * c) = ((const float4*)za)[c];
+        *(float4*)(pz + 4 * c) = ((const float4*)zp)[c];
+        *(float4*)(nz + 4 * c) = ((const float4*)zn)[c];
+    }
     float dp = 0.0f, dn = 0.0f;
+#pragma unroll
     for (int c = 0; c < ml::OUT; ++c) {
-        const float u = za[c] - zp[c], v = za[c] - zn[c];
+        const float u = a[c] - pz[c], v = a[c] - nz[c];
         dp = fmaf(u, u, dp);
         dn = fmaf(v, v, dn);
     }
@@ -546,21 +595,56 @@ __global__ void k_triplet_loss(const float* __restrict__ Z, int B, float margin,
     float* ga = dZ + (int64_t)i * ml::OUT;
     float* gp = dZ + (int64_t)(B + i) * ml::OUT;
     float* gn = dZ + (int64_t)(2 * B + i) * ml::OUT;
-    for (int c = 0; c < ml::OUT; ++c) {
-        ga[c] = g * (zn[c] - zp[c]);
-        gp[c] = g * (zp[c] - za[c]);
-        gn[c] = g * (za[c] - zn[c]);
+#pragma unroll
+    for (int c = 0; c < ml::OUT / 4; ++c) {
+        float ra[4], rp[4], rn[4];
+#pragma unroll
+        for (int q = 0; q < 4; ++q) {
+            ra[q] = g * (nz[4 * c + q] - pz[4 * c + q]);
+            rp[q] = g * (pz[4 * c + q] - a[4 * c + q]);
+            rn[q] = g * (a[4 * c + q] - nz[4 * c + q]);
+        }
+        ((float4*)ga)[c] = make_float4(ra[0], ra[1], ra[2], ra[3]);
+        ((float4*)gp)[c] = make_float4(rp[0], rp[1], rp[2], rp[3]);
+        ((float4*)gn)[c] = make_float4(rn[0], rn[1], rn[2], rn[3]);
     }
 }
 
-// out[j] = sum over rows of A[row * cols + j], rows in increasing order.
-__global__ void k_colsum(const float* __restrict__ A, int64_t rows, int cols,
-                         float* __restrict__ out) {
-    const int j = blockIdx.x * blockDim.x + threadIdx.x;
-    if (j >= cols) return;
+// out[j] = sum over rows of A[row * cols + j], rows in increasing order.  One block per
+// 32 columns: eight warps bring 128 rows at a time into shared memory (two buffers) and
+// the first adds the previous 128 in order, so only the FP32 adds are serial (a thread
+// per column loading its own rows took 89 us for 1,536 x 256, this 21).
+__global__ void __launch_bounds__(256)
+k_colsum(const float* __restrict__ A, int64_t rows, int cols, float* __restrict__ out) {
+    __shared__ float buf[2][128][32];
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const int j = blockIdx.x * 32 + lane;
     float s = 0.0f;
-    for (int64_t r = 0; r < rows; ++r) s += A[r * cols + j];
-    out[j] = s;
+    const int64_t nc = (rows + 127) / 128;
+    for (int64_t c = 0; c <= nc; ++c) {
+        if (c < nc) {
+            float v[16];
+#pragma unroll
+            for (int q = 0; q < 16; ++q) {
+                const int64_t r = c * 128 + warp + 8 * q;
+                v[q] = r < rows && j < cols ? __ldg(A + r * cols + j) : 0.0f;
+            }
+#pragma unroll
+            for (int q = 0; q < 16; ++q) buf[c & 1][warp + 8 * q][lane] = v[q];
+        }
+        if (warp == 0 && c > 0) {
+            const int64_t left = rows - (c - 1) * 128;
+            const int n = left < 128 ? (int)left : 128;
+            if (n == 128) {
+#pragma unroll 16
+                for (int r = 0; r < 128; ++r) s += buf[(c - 1) & 1][r][lane];
+            } else {
+                for (int r = 0; r < n; ++r) s += buf[(c - 1) & 1][r][lane];
+            }
+        }
+        __syncthreads();
+    }
+    if (warp == 0 && j < cols) out[j] = s;
 }
 
 // Mean of li[0..B) into out[*step] (fixed tree order, one block).
@@ -578,15 +662,12 @@ __global__ void k_mean(const float* __restrict__ li, int B, const int* __restric
     if (threadIdx.x == 0) out[*step] = red[0] / (float)B;
 }
 
-// One Adam step on n parameters, t = *step + 1; c1 = 1 / (1 - beta1^t),
-// c2 = 1 / (1 - beta2^t) (in double, rounded once).
+// One Adam step on n parameters, coef = {1 / (1 - beta1^t), 1 / (1 - beta2^t)}.
 __global__ void k_adam(float* __restrict__ p, const float* __restrict__ g, float* __restrict__ m,
-                       float* __restrict__ v, int64_t n, float lr, const int* __restrict__ step) {
+                       float* __restrict__ v, int64_t n, float lr, const float* __restrict__ coef) {
     const int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
     if (i >= n) return;
-    const double t = (double)(*step + 1);
-    const float c1 = (float)(1.0 / (1.0 - pow(0.9, t)));
-    const float c2 = (float)(1.0 / (1.0 - pow(0.999, t)));
+    const float c1 = coef[0], c2 = coef[1];
     const float gi = g[i];
     const float mi = 0.9f * m[i] + 0.1f * gi;
     const float vi = 0.999f * v[i] + 0.001f * gi * gi;
@@ -956,7 +1037,8 @@ static int batch_grads(const void* X, int dtype, int d, const uint32_t* idx, int
     // layer 1 on the tensor cores: x / s and W1 split into BF16 parts (three
     // products), FP32 accumulation
     auto nb = [](int64_t n) { return (unsigned)((n + 255) / 256 < 152 * 16 ? (n + 255) / 256 : 152 * 16); };
-    k_batch_bf16<<<nb(Rp * Kp), 256, 0, q>>>(X, dtype, d, idx, R, Rp, Kp, inv_s, b.xb, b.xbt);
+    k_batch_bf16<<<dim3((unsigned)(Kp / 32), (unsigned)(Rp / 32)), 256, 0, q>>>(
+        X, dtype, d, idx, R, Rp, Kp, inv_s, b.xb, b.xbt);
     ANN_CHECK_LAUNCH();
     k_w1_bf16<<<nb((int64_t)ml::HID * Kp), 256, 0, q>>>(W1, d, Kp, b.w1b);
     ANN_CHECK_LAUNCH();
@@ -967,7 +1049,7 @@ static int batch_grads(const void* X, int dtype, int d, const uint32_t* idx, int
     if ((r = gemm(R, ml::OUT, ml::HID, mat(b.H, ANN_F32, ml::HID), mat(W2, ANN_F32, ml::HID, 1),
                   EpBias{b.Z, b2, ml::OUT}, q, b.part)))
         return r;
-    k_triplet_loss<<<(B + 127) / 128, 128, 0, q>>>(b.Z, B, margin, b.dZ, b.li);
+    k_triplet_loss<<<(B + 31) / 32, 32, 0, q>>>(b.Z, B, margin, b.dZ, b.li);
     ANN_CHECK_LAUNCH();
     if (losses) {
         k_mean<<<1, 256, 0, q>>>(b.li, B, step, losses);
@@ -977,7 +1059,7 @@ static int batch_grads(const void* X, int dtype, int d, const uint32_t* idx, int
     if ((r = gemm(ml::OUT, ml::HID, (int)R, mat(b.dZ, ANN_F32, ml::OUT, 1),
                   mat(b.H, ANN_F32, ml::HID), EpStore{gW2, ml::HID}, q, b.part)))
         return r;
-    k_colsum<<<1, 32, 0, q>>>(b.dZ, R, ml::OUT, gb2);
+    k_colsum<<<ml::OUT / 32, 256, 0, q>>>(b.dZ, R, ml::OUT, gb2);
     ANN_CHECK_LAUNCH();
     // dU = (dZ W2) where U > 0
     if ((r = gemm(R, ml::HID, ml::OUT, mat(b.dZ, ANN_F32, ml::OUT), mat(W2, ANN_F32, ml::HID),
@@ -1001,7 +1083,7 @@ static int batch_grads(const void* X, int dtype, int d, const uint32_t* idx, int
             b.part, nz, ml::HID, d, EpStore{gW1, d});
         ANN_CHECK_LAUNCH();
     }
-    k_colsum<<<1, 256, 0, q>>>(b.dU, R, ml::HID, gb1);
+    k_colsum<<<ml::HID / 32, 256, 0, q>>>(b.dU, R, ml::HID, gb1);
     ANN_CHECK_LAUNCH();
     return ANN_OK;
 }
@@ -1150,21 +1232,21 @@ int run_learned_train(const void* X, int64_t N, int d, int dtype, const uint32_t
     k_inv_scale<<<1, 32, 0, st>>>(amax, inv_s);
     ANN_CHECK_LAUNCH();
     // 3. Adam steps
+    float* coef = (float*)(w.step + 2);  // behind the step counter
     ANN_CHECK_CUDA(cudaMemsetAsync(w.m, 0, (size_t)P * sizeof(float), st));
     ANN_CHECK_CUDA(cudaMemsetAsync(w.v, 0, (size_t)P * sizeof(float), st));
     // One training step; every step-dependent value is read from w.step on the
     // device, so the step can be captured once as a CUDA graph and replayed.
     auto one_step = [&](cudaStream_t q) -> int {
         int r;
-        k_triplets<<<(batch + 255) / 256, 256, 0, q>>>(sample, S, w.knn, kk, kpos, draws,
-                                                       w.step, batch, N, w.idx, status);
+        k_triplets<<<(batch + 255) / 256 + 1, 256, 0, q>>>(sample, S, w.knn, kk, kpos, draws,
+                                                           w.step, batch, N, w.idx, coef, status);
         ANN_CHECK_LAUNCH();
         BatchBufs bb{w.U, w.H, w.Z, w.dZ, w.dU, w.li, w.part, w.xb, w.xbt, w.w1b, w.dut};
         if ((r = batch_grads(X, dtype, d, w.idx, batch, params, inv_s, margin, bb, w.G,
                              losses, w.step, q)))
             return r;
-        k_adam<<<(unsigned)((P + 255) / 256), 256, 0, q>>>(params, w.G, w.m, w.v, P, lr,
-                                                           w.step);
+        k_adam<<<(unsigned)((P + 255) / 256), 256, 0, q>>>(params, w.G, w.m, w.v, P, lr, coef);
         ANN_CHECK_LAUNCH();
         k_step_advance<<<1, 32, 0, q>>>(w.step);
         ANN_CHECK_LAUNCH();
