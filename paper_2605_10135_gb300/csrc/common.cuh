@@ -85,6 +85,32 @@ __device__ __forceinline__ float load_elem(const void* X, int dtype, int64_t i) 
     }
 }
 
+// 16 bytes of a row as floats (V elements of type DT).
+template <int DT>
+struct Chunk16 {
+    static constexpr int V = DT == ANN_F32 ? 4 : (DT == ANN_U8 ? 16 : 8);
+    __device__ static void unpack(const uint4& w, float (&f)[V]) {
+        const uint32_t u[4] = {w.x, w.y, w.z, w.w};
+#pragma unroll
+        for (int i = 0; i < 4; ++i) {
+            if (DT == ANN_F32) {
+                f[i] = __uint_as_float(u[i]);
+            } else if (DT == ANN_F16) {
+                const float2 t = __half22float2(*(const __half2*)&u[i]);
+                f[2 * i] = t.x;
+                f[2 * i + 1] = t.y;
+            } else if (DT == ANN_BF16) {
+                const float2 t = __bfloat1622float2(*(const __nv_bfloat162*)&u[i]);
+                f[2 * i] = t.x;
+                f[2 * i + 1] = t.y;
+            } else {
+#pragma unroll
+                for (int b = 0; b < 4; ++b) f[4 * i + b] = (float)((u[i] >> (8 * b)) & 0xFFu);
+            }
+        }
+    }
+};
+
 __device__ __forceinline__ uint64_t globaltimer() {
     uint64_t t;
     asm volatile("mov.u64 %0, %%globaltimer;" : "=l"(t));
