@@ -3,8 +3,7 @@
 //
 //  distances         : d32 = FP32 squared distance with the terms added in index
 //                      order, unfused (the oracle's definition).  Up to 32
-//                      centroids every d32 is computed (thread per pair); with
-//                      more, the tensor cores screen them first: a tile query keeps the
+//                      centroids every d32 is computed; with more, the tensor cores screen them first: a tile query keeps the
 //                      min(C, r + 6) centroids of smallest tile key per vector,
 //                      and d32 is computed for those only.  The result equals the
 //                      full d32 scan unless more than 6 other centroids lie within
@@ -23,57 +22,97 @@
 
 namespace ann {
 
-// d32 between row `row` of X and centroid c (FP32, index order, unfused).
-__device__ __forceinline__ float d32_row_centroid(const void* X, int dtype, int64_t row, int d,
-                                                  const float* __restrict__ centT, int C, int c) {
-    float s = 0.0f;
-    const int64_t base = row * d;
-    for (int t = 0; t < d; ++t) {
-        float df = __fsub_rn(load_elem(X, dtype, base + t), __ldg(centT + (int64_t)t * C + c));
-        s = __fadd_rn(s, __fmul_rn(df, df));
-    }
-    return s;
+// One more sample of label `lab` (k-means counts), one atomic per label of a warp.
+__device__ __forceinline__ void count_label(int lab, bool valid, int64_t* cnt) {
+    const uint32_t peers = __match_any_sync(0xffffffffu, valid ? lab : -1);
+    if (valid && (threadIdx.x & 31) == __ffs(peers) - 1)
+        atomicAdd((unsigned long long*)(cnt + lab), (unsigned long long)__popc(peers));
 }
 
-// dist[p][c] for p in [p0, p0+np): rows are rowsel[p] (or p itself when NULL).
-__global__ void k_dist_centroids(const void* X, int dtype, int d, const uint32_t* rowsel,
-                                 int64_t p0, int64_t np, const float* __restrict__ centT, int C,
-                                 float* __restrict__ dist) {
-    int64_t total = np * C;
-    for (int64_t q = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; q < total;
-         q += (int64_t)gridDim.x * blockDim.x) {
-        int64_t p = q / C;
-        int c = (int)(q - p * C);
-        int64_t row = rowsel ? (int64_t)rowsel[p0 + p] : p0 + p;
-        dist[q] = d32_row_centroid(X, dtype, row, d, centT, C, c);
-    }
-}
-
-// The r entries of smallest (dist, c) per point, in that order (full scan).
-__global__ void k_topr(const float* __restrict__ dist, int64_t np, int C, int r,
-                       uint32_t* __restrict__ out, int32_t* __restrict__ lab_out,
-                       float* __restrict__ dout) {
-    int64_t p = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
-    if (p >= np) return;
-    const float* dp = dist + p * C;
-    float prev_d = -INFINITY;
-    int prev_c = -1;
-    for (int q = 0; q < r; ++q) {
-        float bd = INFINITY;
-        int bc = -1;
-        for (int c = 0; c < C; ++c) {
-            float v = dp[c];
-            // strictly after (prev_d, prev_c) in (d, c) order
-            bool after = (v > prev_d) || (v == prev_d && c > prev_c);
-            if (!after) continue;
-            if (bc < 0 || v < bd) { bd = v; bc = c; }
+// Up to 32 centroids: d32 (FP32, index order, unfused) of every (row, centroid) pair and
+// the r centroids of smallest (d32, c) per row, in that order.  A block takes 256 RPT / CP
+// rows (CP >= C a power of two), 32 dimensions at a time through shared memory as
+// floats; a thread keeps one centroid and RPT rows: four where the rows fill the chip
+// (a centroid value is read once for four rows, a row value is one broadcast), one below
+// (2,560 rows x 4: 41 us with four, 10 blocks; 15 us with one).  Bound by FP32 issue (3 instructions a
+// pair and dimension); a thread per pair with element loads and a distance array took
+// 1.29 ms for 1M x 16 x 128 uint8 and 2.65 ms for 200k x 16 x 1024 FP16, this 0.50 ms and 0.98 ms.
+// Rows p0 .. p0 + np - 1 (through rowsel when given); out, lab_out, dout, cnt optional.
+template <int DT, int RPT>
+__global__ void __launch_bounds__(256)
+k_assign_small(const void* X, int d, const uint32_t* __restrict__ rowsel, int64_t p0, int64_t np,
+               const float* __restrict__ centT, int C, int cp, int r, uint32_t* __restrict__ out,
+               int32_t* __restrict__ lab_out, float* __restrict__ dout, int64_t* cnt) {
+    constexpr int TT = 32;
+    extern __shared__ float asm_[];
+    const int RB = 256 * RPT / cp, rg_n = 256 / cp;  // rows of a block, row groups
+    float* xs = asm_;                            // [RB][TT + 1]
+    float* cs = xs + RB * (TT + 1);              // [TT][cp]
+    float* ds = cs + TT * cp;                    // [RB][cp + 1]
+    const int tid = threadIdx.x, c = tid % cp, rg = tid / cp;
+    const int64_t b0 = (int64_t)blockIdx.x * RB;
+    const int lane = tid & 31, warp = tid >> 5;
+    float acc[RPT];
+#pragma unroll
+    for (int i = 0; i < RPT; ++i) acc[i] = 0.0f;
+    for (int t0 = 0; t0 < d; t0 += TT) {
+        const int nt = d - t0 < TT ? d - t0 : TT;
+#pragma unroll 8
+        for (int rr = warp; rr < RB; rr += 8) {  // a warp loads 32 dimensions of a row
+            const int64_t p = b0 + rr;
+            float v = 0.0f;
+            if (p < np && lane < nt) {
+                const int64_t row = rowsel ? (int64_t)__ldg(rowsel + p0 + p) : p0 + p;
+                v = load_elem(X, DT, row * d + t0 + lane);
+            }
+            xs[rr * (TT + 1) + lane] = v;
         }
-        if (bc < 0) bc = 0;  // unreachable for finite distances
-        if (out) out[p * r + q] = (uint32_t)bc;
-        if (dout) dout[p * r + q] = bd;
-        if (lab_out && q == 0) lab_out[p] = bc;
-        prev_d = bd;
-        prev_c = bc;
+        for (int e = tid; e < TT * cp; e += 256) {
+            const int t = e / cp, cc = e % cp;
+            cs[e] = t < nt && cc < C ? __ldg(centT + (int64_t)(t0 + t) * C + cc) : 0.0f;
+        }
+        __syncthreads();
+        const float* x0 = xs + rg * (TT + 1);
+        const int rs = rg_n * (TT + 1);
+#pragma unroll 4
+        for (int t = 0; t < nt; ++t) {
+            const float cv = cs[t * cp + c];
+#pragma unroll
+            for (int i = 0; i < RPT; ++i) {
+                const float df = __fsub_rn(x0[i * rs + t], cv);
+                acc[i] = __fadd_rn(acc[i], __fmul_rn(df, df));
+            }
+        }
+        __syncthreads();
+    }
+#pragma unroll
+    for (int i = 0; i < RPT; ++i) ds[(rg + i * rg_n) * (cp + 1) + c] = acc[i];
+    __syncthreads();
+    for (int rr = tid; rr < (RB + 31) / 32 * 32; rr += 256) {  // whole warps
+        const int64_t p = b0 + rr;
+        const bool in = rr < RB && p < np;
+        const float* dp = ds + (rr < RB ? rr : 0) * (cp + 1);
+        float prev_d = -INFINITY;
+        int prev_c = -1, first = 0;
+        for (int q = 0; q < r; ++q) {
+            float bd = INFINITY;
+            int bc = -1;
+            for (int k = 0; k < C; ++k) {
+                const float v = dp[k];
+                // strictly after (prev_d, prev_c) in (d, c) order
+                const bool after = (v > prev_d) || (v == prev_d && k > prev_c);
+                if (!after) continue;
+                if (bc < 0 || v < bd) { bd = v; bc = k; }
+            }
+            if (bc < 0) bc = 0;  // unreachable for finite distances
+            if (in && out) out[p * r + q] = (uint32_t)bc;
+            if (in && dout) dout[p * r + q] = bd;
+            if (q == 0) first = bc;
+            prev_d = bd;
+            prev_c = bc;
+        }
+        if (in && lab_out) lab_out[p] = first;
+        if (cnt) count_label(first, in, cnt);
     }
 }
 
@@ -130,9 +169,12 @@ __global__ void k_d32_cand_f4(const float* __restrict__ X, int d, const uint32_t
 // The r candidates of smallest (d32, centroid id) per point, in that order.
 __global__ void k_topr_cand(const float* __restrict__ dist, const uint32_t* __restrict__ cand,
                             int64_t np, int ks, int r, uint32_t* __restrict__ out,
-                            int32_t* __restrict__ lab_out, float* __restrict__ dout) {
-    const int64_t p = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
-    if (p >= np) return;
+                            int32_t* __restrict__ lab_out, float* __restrict__ dout,
+                            int64_t* cnt) {
+    const int64_t p0 = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
+    const bool in = p0 < np;
+    const int64_t p = in ? p0 : np - 1;  // (whole warps reach the count below)
+    int first = 0;
     const float* dp = dist + p * ks;
     const uint32_t* cp = cand + p * ks;
     float prev_d = -INFINITY;
@@ -151,101 +193,151 @@ __global__ void k_topr_cand(const float* __restrict__ dist, const uint32_t* __re
             }
         }
         if (bc < 0) bc = 0;  // unreachable: ks >= r distinct candidates
-        if (out) out[p * r + q] = (uint32_t)bc;
-        if (dout) dout[p * r + q] = bd;
-        if (lab_out && q == 0) lab_out[p] = (int32_t)bc;
+        if (in && out) out[p * r + q] = (uint32_t)bc;
+        if (in && dout) dout[p * r + q] = bd;
+        if (q == 0) first = (int)bc;
         prev_d = bd;
         prev_c = bc;
     }
+    if (in && lab_out) lab_out[p] = first;
+    if (cnt) count_label(first, in, cnt);
 }
 
 // FP64 centroid sums in sample order (so each (c, t) sum is the plain sequential
 // one).  list[off[c] .. off[c] + cnt[c]) holds the rows of the samples labelled c
-// in sample order; one warp per (c, 32 consecutive dimensions) keeps a register
-// accumulator per lane, visits only its own samples, loads 8 rows ahead, and only
-// the FP64 adds are serial.  The C x d/32 warps are independent.
-__global__ void k_kmeans_sums_lists(const void* X, int dtype, int d,
-                                    const uint32_t* __restrict__ list,
-                                    const int64_t* __restrict__ off,
-                                    const int64_t* __restrict__ cnt, int C,
-                                    double* __restrict__ sums) {
-    const int lane = threadIdx.x & 31;
-    const int64_t w = (blockIdx.x * (int64_t)blockDim.x + threadIdx.x) >> 5;
+// in sample order; one block per (c, 32 consecutive dimensions).  Its warps take turns
+// at bringing 64 rows into shared memory (KSR rows a buffer, KSB buffers in flight) and
+// warp 0 adds them in order, so only the FP64 adds are serial: a warp that loaded its
+// own rows, 8 at a time, paid a list and a row access for every 8 adds (892 us for
+// the largest of 16 clusters of 10,000 samples, now 80 us; the largest of 11 of 2,816 BF16 rows 340 -> 49).
+// The adder widens its values to double by their bits (the FP64 pipe takes about 64
+// clocks a warp for a conversion as for an add), except in a buffer that its filling
+// warp marked for holding subnormal or non-finite values; uint8 sums are kept as
+// integers, which FP64 would hold exactly.
+constexpr int KSR = 64, KSB = 4;
+template <int DT> struct SumElem {
+    using T = float;
+    using A = double;
+    __device__ static T of(const void* X, int64_t i) { return load_elem(X, DT, i); }
+    __device__ static bool odd(T v) {  // not zero and not normal
+        const uint32_t a = __float_as_uint(v) & 0x7FFFFFFFu;
+        return a != 0 && a - 0x00800000u >= 0x7F000000u;
+    }
+    __device__ static A add(A a, T v) { return __dadd_rn(a, (double)v); }
+    __device__ static A add_plain(A acc, T v) {  // zero or normal
+        const uint32_t u = __float_as_uint(v), a = u & 0x7FFFFFFFu;
+        const uint32_t hi = (u & 0x80000000u) | (a ? (a >> 3) + 0x38000000u : 0u);
+        return __dadd_rn(acc, __hiloint2double((int)hi, (int)(a << 29)));
+    }
+};
+template <> struct SumElem<ANN_U8> {
+    using T = uint8_t;
+    using A = unsigned long long;
+    __device__ static T of(const void* X, int64_t i) { return __ldg((const uint8_t*)X + i); }
+    __device__ static bool odd(T) { return false; }
+    __device__ static A add(A a, T v) { return a + v; }
+    __device__ static A add_plain(A a, T v) { return a + v; }
+};
+
+template <int DT>
+__global__ void __launch_bounds__(32 * (KSB + 1))
+k_kmeans_sums_lists(const void* X, int d, const uint32_t* __restrict__ list,
+                    const int64_t* __restrict__ off, const int64_t* __restrict__ cnt, int C,
+                    float* __restrict__ cent, float* __restrict__ centT) {
+    using E = typename SumElem<DT>::T;
+    __shared__ E buf[KSB][KSR][32];
+    __shared__ bool odd[KSB];
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     const int nt = (d + 31) / 32;
-    if (w >= (int64_t)C * nt) return;
-    const int c = (int)(w / nt);
-    const int t = (int)(w % nt) * 32 + lane;
+    const int c = blockIdx.x / nt;
+    const int t = (blockIdx.x % nt) * 32 + lane;
     const bool active = t < d;
     const uint32_t* lc = list + off[c];
     const int64_t n = cnt[c];
-    double acc = 0.0;
-    for (int64_t i0 = 0; i0 < n; i0 += 8) {
-        float v[8];
+    typename SumElem<DT>::A acc = 0;
+    // round g: warp 1 + b fills buffer b with rows (g KSB + b) KSR ..., warp 0 adds the
+    // buffers of round g - 1 meanwhile (kept in registers until the barrier)
+    const int64_t rounds = (n + (int64_t)KSR * KSB - 1) / (KSR * KSB);
+    for (int64_t g = 0; g <= rounds; ++g) {
+        E v[KSR];
+        const int64_t i0 = (g * KSB + warp - 1) * KSR;
+        if (warp > 0 && g < rounds) {
+            const uint32_t r0 = i0 + lane < n ? __ldg(lc + i0 + lane) : 0u;
+            const uint32_t r1 = i0 + 32 + lane < n ? __ldg(lc + i0 + 32 + lane) : 0u;
 #pragma unroll
-        for (int u = 0; u < 8; ++u)
-            v[u] = (active && i0 + u < n) ? load_elem(X, dtype, (int64_t)__ldg(lc + i0 + u) * d + t)
-                                          : 0.0f;
+            for (int u = 0; u < KSR; ++u) {
+                const uint32_t row = __shfl_sync(0xffffffffu, u < 32 ? r0 : r1, u & 31);
+                v[u] = active && i0 + u < n ? SumElem<DT>::of(X, (int64_t)row * d + t)
+                                            : E(0);
+            }
+        }
+        if (warp == 0 && g > 0) {
+            for (int b = 0; b < KSB; ++b) {
+                const int64_t left = n - ((g - 1) * KSB + b) * KSR;
+                const int m = left >= KSR ? KSR : (int)left;
+                if (m == KSR && !odd[b]) {
+#pragma unroll 16
+                    for (int u = 0; u < KSR; ++u) acc = SumElem<DT>::add_plain(acc, buf[b][u][lane]);
+                } else {
+                    for (int u = 0; u < m; ++u) acc = SumElem<DT>::add(acc, buf[b][u][lane]);
+                }
+            }
+        }
+        __syncthreads();  // the round before is summed
+        if (warp > 0 && g < rounds) {
+            bool o = false;
 #pragma unroll
-        for (int u = 0; u < 8; ++u)
-            if (i0 + u < n) acc = __dadd_rn(acc, (double)v[u]);
+            for (int u = 0; u < KSR; ++u) {
+                buf[warp - 1][u][lane] = v[u];
+                o = o || SumElem<DT>::odd(v[u]);
+            }
+            o = __any_sync(0xffffffffu, o);
+            if (lane == 0) odd[warp - 1] = o;
+        }
+        __syncthreads();
     }
-    if (active) sums[(int64_t)c * d + t] = acc;
+    // the mean, rounded to float once; an empty cluster keeps its centroid
+    if (warp == 0 && active && n > 0) {
+        const float v = (float)__ddiv_rn((double)acc, (double)n);
+        cent[(int64_t)c * d + t] = v;
+        centT[(int64_t)t * C + c] = v;
+    }
 }
 
-// Exclusive prefix of the label counts (C <= 1024; one thread).
-__global__ void k_label_offsets(const int64_t* __restrict__ cnt, int C, int64_t* __restrict__ off) {
-    if (threadIdx.x || blockIdx.x) return;
-    int64_t a = 0;
-    for (int c = 0; c < C; ++c) {
-        off[c] = a;
-        a += cnt[c];
-    }
-    off[C] = a;
-}
-
-// Rows of the samples labelled c in sample order (one block of 256 per c).
-__global__ void __launch_bounds__(256)
+// Rows of the samples labelled c in sample order (one block of 1024 per c), and off[c],
+// the number of samples with smaller labels.
+__global__ void __launch_bounds__(1024)
     k_label_lists(const int32_t* __restrict__ lab, const uint32_t* __restrict__ sample,
-                  int64_t S, const int64_t* __restrict__ off, uint32_t* __restrict__ list) {
-    __shared__ int wcnt[8];
-    __shared__ int64_t run;
+                  int64_t S, const int64_t* __restrict__ cnt, int64_t* __restrict__ off,
+                  uint32_t* __restrict__ list) {
+    __shared__ int wcnt[2][32];
     const int c = blockIdx.x;
     const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
-    if (threadIdx.x == 0) run = 0;
+    // S < 2^32: 32-bit sums of each warp, then over the warps in 64 bits
+    __shared__ unsigned long long base_s;
+    if (threadIdx.x == 0) base_s = 0;
     __syncthreads();
-    for (int64_t s0 = 0; s0 < S; s0 += 256) {
+    unsigned long long mine = 0;
+    for (int q = threadIdx.x; q < c; q += blockDim.x) mine += (unsigned long long)cnt[q];
+    for (int o = 16; o; o >>= 1) mine += __shfl_xor_sync(0xffffffffu, mine, o);
+    if (lane == 0 && mine) atomicAdd(&base_s, mine);
+    __syncthreads();
+    const int64_t base = (int64_t)base_s;
+    if (threadIdx.x == 0) off[c] = base;
+    int64_t run = base;
+    int buf = 0;
+    for (int64_t s0 = 0; s0 < S; s0 += 1024, buf ^= 1) {
         const int64_t s = s0 + threadIdx.x;
         const bool f = s < S && lab[s] == c;
         const uint32_t b = __ballot_sync(0xffffffffu, f);
-        if (lane == 0) wcnt[wid] = __popc(b);
-        __syncthreads();
-        int before = 0, total = 0;
-        for (int q = 0; q < 8; ++q) {
-            if (q < wid) before += wcnt[q];
-            total += wcnt[q];
-        }
-        if (f) list[off[c] + run + before + __popc(b & ((1u << lane) - 1))] = sample[s];
-        __syncthreads();
-        if (threadIdx.x == 0) run += total;
-        __syncthreads();
+        if (lane == 0) wcnt[buf][wid] = __popc(b);
+        __syncthreads();  // (two buffers: the next turn's counts go to the other one)
+        const int wc = wcnt[buf][lane];
+        const int before = __reduce_add_sync(0xffffffffu, lane < wid ? wc : 0);
+        const int total = __reduce_add_sync(0xffffffffu, wc);
+        if (f) list[run + before + __popc(b & ((1u << lane) - 1))] = sample[s];
+        run += total;
     }
-}
-
-__global__ void k_count_labels(const int32_t* __restrict__ lab, int64_t S, int64_t* cnt) {
-    for (int64_t s = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; s < S;
-         s += (int64_t)gridDim.x * blockDim.x)
-        atomicAdd((unsigned long long*)(cnt + lab[s]), 1ull);
-}
-
-__global__ void k_kmeans_update(const double* __restrict__ sums, const int64_t* __restrict__ cnt,
-                                int C, int d, float* __restrict__ cent, float* __restrict__ centT) {
-    int64_t q = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
-    if (q >= (int64_t)C * d) return;
-    int c = (int)(q / d), t = (int)(q - (int64_t)c * d);
-    float v = cent[q];
-    if (cnt[c] > 0) v = (float)__ddiv_rn(sums[q], (double)cnt[c]);
-    cent[q] = v;
-    centT[(int64_t)t * C + c] = v;
 }
 
 __global__ void k_transpose_cent(const float* __restrict__ cent, int C, int d, float* cent_out,
@@ -375,11 +467,10 @@ size_t partition_ws(int64_t N, int d, int C, int r, int64_t S, PartitionWs* out,
     w.centT = cv.take<float>((size_t)C * d);
     const bool full = C <= FULL_SCAN_C;
     if (full) w.sws_bytes = 0;
-    w.dist = cv.take<float>((size_t)w.chunk * (full ? C : w.ks));
-    w.cand = cv.take<uint32_t>((size_t)w.chunk * w.ks);
+    w.dist = full ? nullptr : cv.take<float>((size_t)w.chunk * w.ks);
+    w.cand = full ? nullptr : cv.take<uint32_t>((size_t)w.chunk * w.ks);
     w.sws = cv.take<uint8_t>(w.sws_bytes + 1);
     w.lab = cv.take<int32_t>((size_t)(S > 0 ? S : 1));
-    w.sums = cv.take<double>((size_t)C * d);
     w.cnt = cv.take<int64_t>((size_t)C);
     w.loff = cv.take<int64_t>((size_t)C + 1);
     w.llist = cv.take<uint32_t>((size_t)(S > 0 ? S : 1));
@@ -394,13 +485,22 @@ size_t partition_ws(int64_t N, int d, int C, int r, int64_t S, PartitionWs* out,
 // when given): tensor-core screen, then d32 of the candidates.
 static int assign_chunk(const void* X, int dtype, int d, const uint32_t* rowsel, int64_t p0,
                         int64_t np, int C, int r, const PartitionWs& w, uint32_t* out,
-                        int32_t* lab, cudaStream_t st, float* dout = nullptr) {
+                        int32_t* lab, cudaStream_t st, float* dout = nullptr,
+                        int64_t* cnt = nullptr) {
     if (C <= FULL_SCAN_C) {
-        const int64_t tot = np * C;
-        const unsigned g = (unsigned)((tot + 255) / 256 < 65535 * 8 ? (tot + 255) / 256 : 65535 * 8);
-        k_dist_centroids<<<g, 256, 0, st>>>(X, dtype, d, rowsel, p0, np, w.centT, C, w.dist);
-        ANN_CHECK_LAUNCH();
-        k_topr<<<(unsigned)((np + 255) / 256), 256, 0, st>>>(w.dist, np, C, r, out, lab, dout);
+        int cp = 4;
+        while (cp < C) cp <<= 1;
+        const bool four = np * cp >= 152 * 1024;  // a block of four rows a thread per SM
+        const int rb = 256 * (four ? 4 : 1) / cp;
+        const size_t sm = ((size_t)rb * 33 + 32 * cp + (size_t)rb * (cp + 1)) * sizeof(float);
+#define ANN_ASSIGN(DT) (four ? k_assign_small<DT, 4> : k_assign_small<DT, 1>)
+        const auto kern = dtype == ANN_F32   ? ANN_ASSIGN(ANN_F32)
+                          : dtype == ANN_F16  ? ANN_ASSIGN(ANN_F16)
+                          : dtype == ANN_BF16 ? ANN_ASSIGN(ANN_BF16)
+                                              : ANN_ASSIGN(ANN_U8);
+#undef ANN_ASSIGN
+        kern<<<(unsigned)((np + rb - 1) / rb), 256, sm, st>>>(X, d, rowsel, p0, np, w.centT, C, cp,
+                                                             r, out, lab, dout, cnt);
         ANN_CHECK_LAUNCH();
         return ANN_OK;
     }
@@ -417,7 +517,7 @@ static int assign_chunk(const void* X, int dtype, int d, const uint32_t* rowsel,
         k_d32_cand<<<g, 256, 0, st>>>(X, dtype, d, rowsel, p0, np, w.cent, w.cand, ks, w.dist);
     ANN_CHECK_LAUNCH();
     k_topr_cand<<<(unsigned)((np + 255) / 256), 256, 0, st>>>(w.dist, w.cand, np, ks, r, out, lab,
-                                                               dout);
+                                                               dout, cnt);
     ANN_CHECK_LAUNCH();
     return ANN_OK;
 }
@@ -433,26 +533,23 @@ static int kmeans_stage(const void* X, int d, int dtype, int C, const float* ini
     k_transpose_cent<<<nb(cd, tpb), tpb, 0, st>>>(init_centroids, C, d, w.cent, w.centT);
     ANN_CHECK_LAUNCH();
     for (int it = 0; it < iters && S > 0; ++it) {
+        ANN_CHECK_CUDA(cudaMemsetAsync(w.cnt, 0, sizeof(int64_t) * C, st));
         for (int64_t p0 = 0; p0 < S; p0 += w.chunk) {
             int64_t np = S - p0 < w.chunk ? S - p0 : w.chunk;
             int rc = assign_chunk(X, dtype, d, sample_idx, p0, np, C, 1, w, nullptr,
-                                  w.lab + p0, st);
+                                  w.lab + p0, st, nullptr, w.cnt);
             if (rc) return rc;
         }
-        ANN_CHECK_CUDA(cudaMemsetAsync(w.cnt, 0, sizeof(int64_t) * C, st));
-        k_count_labels<<<nb(S, tpb) < 4096u ? nb(S, tpb) : 4096u, tpb, 0, st>>>(w.lab, S, w.cnt);
-        ANN_CHECK_LAUNCH();
-        k_label_offsets<<<1, 32, 0, st>>>(w.cnt, C, w.loff);
-        ANN_CHECK_LAUNCH();
-        k_label_lists<<<C, 256, 0, st>>>(w.lab, sample_idx, S, w.loff, w.llist);
+        k_label_lists<<<C, 1024, 0, st>>>(w.lab, sample_idx, S, w.cnt, w.loff, w.llist);
         ANN_CHECK_LAUNCH();
         {
-            const int64_t warps = (int64_t)C * ((d + 31) / 32);
-            k_kmeans_sums_lists<<<(unsigned)((warps + 3) / 4), 128, 0, st>>>(
-                X, dtype, d, w.llist, w.loff, w.cnt, C, w.sums);
+            const unsigned g = (unsigned)(C * ((d + 31) / 32));
+            const auto sums = dtype == ANN_F32   ? k_kmeans_sums_lists<ANN_F32>
+                              : dtype == ANN_F16  ? k_kmeans_sums_lists<ANN_F16>
+                              : dtype == ANN_BF16 ? k_kmeans_sums_lists<ANN_BF16>
+                                                  : k_kmeans_sums_lists<ANN_U8>;
+            sums<<<g, 32 * (KSB + 1), 0, st>>>(X, d, w.llist, w.loff, w.cnt, C, w.cent, w.centT);
         }
-        ANN_CHECK_LAUNCH();
-        k_kmeans_update<<<nb(cd, tpb), tpb, 0, st>>>(w.sums, w.cnt, C, d, w.cent, w.centT);
         ANN_CHECK_LAUNCH();
     }
     ANN_CHECK_CUDA(cudaMemcpyAsync(centroids_out, w.cent, sizeof(float) * cd,

@@ -12,13 +12,12 @@ namespace ann {
 struct PartitionWs {
     float* cent;       // [C*d] working centroids
     float* centT;      // [d*C] transposed copy read by the distance kernel
-    float* dist;       // [chunk*C] (full scan) or [chunk*ks] d32 of the screened candidates
-    uint32_t* cand;    // [chunk*ks] screened centroid ids
+    float* dist;       // [chunk*ks] d32 of the screened candidates (NULL: full scan)
+    uint32_t* cand;    // [chunk*ks] screened centroid ids (NULL: full scan)
     uint8_t* sws;      // screening workspace
     size_t sws_bytes;
     int ks;            // screened centroids per vector (final assignment)
     int32_t* lab;      // [S]
-    double* sums;      // [C*d]
     int64_t* cnt;      // [C]
     int64_t* loff;     // [C+1] offsets of the per-label sample lists
     uint32_t* llist;   // [S] sample rows grouped by label, sample order inside a label
