@@ -1476,8 +1476,133 @@ __global__ void __launch_bounds__(1024)
     }
 }
 
-static int launch_pivot_chain(const void* X, int dtype, int d, const KnnWs& w, int C,
-                              cudaStream_t st) {
+// The same chain in two kernels where a scratch matrix is at hand: all pivot distances
+// first (64 x 64 tiles, 4 x 4 a thread, 32 dimensions at a time), then one warp per
+// shard walks the chain, a step being up to 32 independent loads a lane of the current
+// pivot's row and two warp minima.  One block per shard that scored every pivot in each
+// step took 5.5 us a step (5.5 ms for 16 shards of 125k uint8 rows, d = 128); now
+// 0.92 ms in all.  Row q of shard s is row offsets[s] / 128 + s + q of the matrix (a
+// shard has at most n / 128 + 1 pivots, so shards do not meet); its pitch is 1,024.
+// (-1 where inconsistent offsets, reported elsewhere, would leave the matrix.)
+__device__ __forceinline__ int64_t pivot_row0(const int64_t* offsets, int s, int P, int64_t nrows) {
+    const int64_t r = offsets[s] / kt::CELL + s;
+    return offsets[s] >= 0 && r + P <= nrows ? r : -1;
+}
+
+template <int DT>
+__global__ void __launch_bounds__(256)
+k_pivot_dist(const void* X, int d, const int64_t* __restrict__ psrc,
+             const int64_t* __restrict__ offsets, const int64_t* __restrict__ ppad_off,
+             const int32_t* __restrict__ npiv, int64_t nrows, float* __restrict__ mat) {
+    __shared__ float As[32][65], Bs[32][65];
+    const int s = blockIdx.z, P = npiv[s];
+    const int a0 = blockIdx.x * 64, b0 = blockIdx.y * 64;
+    const int64_t row0 = pivot_row0(offsets, s, P, nrows);
+    if (a0 >= P || b0 >= P || row0 < 0) return;
+    const int64_t base = ppad_off[s];
+    const int tid = threadIdx.x, tx = tid & 15, ty = tid >> 4, lane = tid & 31, warp = tid >> 5;
+    float acc[4][4] = {};
+    for (int t0 = 0; t0 < d; t0 += 32) {
+        const bool in = t0 + lane < d;
+#pragma unroll
+        for (int q = 0; q < 8; ++q) {  // a warp loads 32 dimensions of a row
+            const int r = warp + 8 * q;
+            const int64_t ra = a0 + r < P ? psrc[base + a0 + r] : -1;
+            const int64_t rb = b0 + r < P ? psrc[base + b0 + r] : -1;
+            As[lane][r] = in && ra >= 0 ? load_elem(X, DT, ra * d + t0 + lane) : 0.0f;
+            Bs[lane][r] = in && rb >= 0 ? load_elem(X, DT, rb * d + t0 + lane) : 0.0f;
+        }
+        __syncthreads();
+#pragma unroll 8
+        for (int t = 0; t < 32; ++t) {
+            float a[4], b[4];
+#pragma unroll
+            for (int i = 0; i < 4; ++i) {
+                a[i] = As[t][ty + 16 * i];
+                b[i] = Bs[t][tx + 16 * i];
+            }
+#pragma unroll
+            for (int i = 0; i < 4; ++i)
+#pragma unroll
+                for (int j = 0; j < 4; ++j) {
+                    const float df = a[i] - b[j];
+                    acc[i][j] = fmaf(df, df, acc[i][j]);
+                }
+        }
+        __syncthreads();
+    }
+    float* m = mat + row0 * 1024;
+#pragma unroll
+    for (int i = 0; i < 4; ++i)
+#pragma unroll
+        for (int j = 0; j < 4; ++j) {
+            const int a = a0 + ty + 16 * i, b = b0 + tx + 16 * j;
+            if (a < P && b < P) m[(int64_t)a * 1024 + b] = acc[i][j];
+        }
+}
+
+__global__ void __launch_bounds__(32)
+k_pivot_walk(const int64_t* __restrict__ offsets, const int64_t* __restrict__ ppad_off,
+             const int32_t* __restrict__ npiv, int64_t nrows, const float* __restrict__ mat,
+             uint32_t* __restrict__ crank) {
+    const int s = blockIdx.x, P = npiv[s], lane = threadIdx.x;
+    const int64_t row0 = pivot_row0(offsets, s, P, nrows);
+    const float* m = mat + row0 * 1024;
+    uint32_t* rank = crank + ppad_off[s];
+    if (row0 < 0) {
+        for (int q = lane; q < P; q += 32) rank[q] = (uint32_t)q;
+        return;
+    }
+    // bit i: pivot lane + 32 i is taken or missing
+    uint32_t taken = 0;
+    for (int i = 0; i < 32; ++i)
+        if (lane + 32 * i >= P) taken |= 1u << i;
+    int cur = 0;
+    for (int step = 0; step < P; ++step) {
+        if ((cur & 31) == lane) taken |= 1u << (cur >> 5);
+        if (lane == 0) rank[cur] = (uint32_t)step;
+        const float* row = m + (int64_t)cur * 1024 + lane;
+        uint32_t best = 0xFFFFFFFFu, at = 0xFFFFFFFFu;
+        uint32_t v[32];
+#pragma unroll
+        for (int i = 0; i < 32; ++i)  // (all loads before the first use)
+            v[i] = (taken >> i) & 1u ? 0xFFFFFFFFu : __float_as_uint(__ldg(row + 32 * i));
+#pragma unroll
+        for (int i = 0; i < 32; ++i)  // squared distances: their bits order them
+            if (v[i] < best) {
+                best = v[i];
+                at = lane + 32 * i;
+            }
+        const uint32_t lo = __reduce_min_sync(0xffffffffu, best);
+        const uint32_t nx = __reduce_min_sync(0xffffffffu, best == lo ? at : 0xFFFFFFFFu);
+        if (nx >= (uint32_t)P) {  // the last step, or distances that are not numbers
+            if (step + 1 == P) break;
+            const uint32_t fr = ~taken;  // the free pivot of smallest index
+            cur = (int)__reduce_min_sync(0xffffffffu, fr ? lane + 32 * (__ffs(fr) - 1) : 0xFFFFFFFFu);
+        } else {
+            cur = (int)nx;
+        }
+    }
+}
+
+static int launch_pivot_chain(const void* X, int dtype, int d, const int64_t* offsets,
+                              const KnnWs& w, int C, int cell, cudaStream_t st) {
+    if (w.tlist && cell == kt::CELL) {  // the tile lists are written later
+        float* mat = (float*)w.tlist;
+        const dim3 g(16, 16, (unsigned)C);
+#define ANN_PDIST(DT) k_pivot_dist<DT><<<g, 256, 0, st>>>(X, d, w.psrc, offsets, w.ppad_off, w.npiv, w.nblocks, mat)
+        switch (dtype) {
+        case ANN_F32: ANN_PDIST(ANN_F32); break;
+        case ANN_F16: ANN_PDIST(ANN_F16); break;
+        case ANN_BF16: ANN_PDIST(ANN_BF16); break;
+        default: ANN_PDIST(ANN_U8); break;
+        }
+#undef ANN_PDIST
+        ANN_CHECK_LAUNCH();
+        k_pivot_walk<<<C, 32, 0, st>>>(offsets, w.ppad_off, w.npiv, w.nblocks, mat, w.crank);
+        ANN_CHECK_LAUNCH();
+        return ANN_OK;
+    }
     const bool vec = ((size_t)d * dtype_bytes(dtype)) % 16 == 0 && (uintptr_t)X % 16 == 0;
     const size_t sm = (size_t)d * sizeof(float);
 #define ANN_CHAIN(DT)                                                                          \
@@ -1556,6 +1681,25 @@ __global__ void k_rowmap_cells(const uint32_t* __restrict__ members,
         gid[pr] = v >= 0 ? (uint32_t)v : ANN_PAD;
         outrow[pr] = orow;
     }
+}
+
+// s + sum of (a[t] - b[t])^2 in index order, unfused: differences and squares two at a
+// time (packed FP32 pairs round like two scalar operations), the additions one by one.
+template <int V>
+__device__ __forceinline__ float sq_diff_add(const float (&a)[V], const float (&b)[V], float s) {
+#pragma unroll
+    for (int t = 0; t < V; t += 2) {
+        uint64_t pa, pb, d;
+        asm("mov.b64 %0, {%1, %2};" : "=l"(pa) : "f"(a[t]), "f"(a[t + 1]));
+        asm("mov.b64 %0, {%1, %2};" : "=l"(pb) : "f"(-b[t]), "f"(-b[t + 1]));
+        asm("add.rn.f32x2 %0, %1, %2;" : "=l"(d) : "l"(pa), "l"(pb));
+        asm("mul.rn.f32x2 %0, %1, %1;" : "=l"(d) : "l"(d));
+        float q0, q1;
+        asm("mov.b64 {%0, %1}, %2;" : "=f"(q0), "=f"(q1) : "l"(d));
+        s = __fadd_rn(s, q0);
+        s = __fadd_rn(s, q1);
+    }
+    return s;
 }
 
 // ---- exact re-rank (FP32 direct form) -------------------------------------------
@@ -1640,6 +1784,23 @@ k_pool_finalize(const KnnParams P) {
         Bound T;
         T.key = T.id = 0xFFFFFFFFu;
         if (n > kp) T = warp_select(v, n, kp, kp, gidrow);
+        if (!P.out_d && !P.split_list) {
+            // re-ranked lists: their order decides nothing, so the kept entries go out as
+            // they come (the sort below and its staging are about half of this kernel)
+            const int64_t orow = P.outrow ? P.outrow[pr.a_row0 + i] : pr.out_row0 + i;
+            uint32_t* out = P.out_id + orow * P.k_out;
+            int at = 0;
+#pragma unroll
+            for (int e = 0; e < 2 * EH; ++e) {
+                const bool keep = bound_keeps(T, v[e], gidrow);
+                const uint32_t b = __ballot_sync(0xffffffffu, keep);
+                const int pos = at + __popc(b & ((1u << lane) - 1u));
+                if (keep && pos < P.k_out) out[pos] = pr.id0 + column_gid(gidrow, (uint32_t)v[e]);
+                at += __popc(b);
+            }
+            for (int e = at + lane; e < P.k_out; e += 32) out[e] = ANN_PAD;
+            continue;
+        }
         // the kept entries (kp of them, or all n) into the staging array
         for (int e = lane; e < 32 * KE; e += 32) stg[e] = ~0ull;
         __syncwarp();
@@ -1683,7 +1844,7 @@ k_pool_finalize(const KnnParams P) {
                     dd = fmaf(2.0f, ord2f((uint32_t)(w[e] >> 32)), nx);
                 }
                 P.out_id[orow * P.k_out + slot] = id;
-                if (P.out_d) P.out_d[orow * P.k_out + slot] = dd;
+                P.out_d[orow * P.k_out + slot] = dd;
             }
         }
     }
@@ -1759,8 +1920,11 @@ k_split_merge(const uint64_t* __restrict__ lists, int ns, int64_t stride, int kp
     }
 }
 
-template <int E>
-__global__ void k_rerank(const void* X, const void* Xrow, int dtype, int d,
+// Four candidates are scored per pass so that their loads overlap (one at a time with a
+// type switch per element took 2.33 ms for 233k rows of 64 candidates, d = 50 BF16; this
+// 0.97 ms).
+template <int E, int DT>
+__global__ void k_rerank(const void* X, const void* Xrow, int d,
                          const uint32_t* __restrict__ row_ids, int64_t nrows,
                          const uint32_t* __restrict__ cand, int kc, int k,
                          uint32_t* __restrict__ out_id, float* __restrict__ out_d,
@@ -1773,21 +1937,37 @@ __global__ void k_rerank(const void* X, const void* Xrow, int dtype, int d,
     uint64_t keys[E];
 #pragma unroll
     for (int e = 0; e < E; ++e) keys[e] = ~0ull;
-    for (int c = 0; c < kc; ++c) {
-        const uint32_t v = cand[p * kc + c];
-        if (v == ANN_PAD) continue;  // uniform
-        float s = 0.0f;
-        for (int t = lane; t < d; t += 32) {
-            const float df = __fsub_rn(load_elem(Xrow, dtype, u * d + t),
-                                       load_elem(X, dtype, (int64_t)v * d + t));
-            s = __fadd_rn(s, __fmul_rn(df, df));
-        }
-        for (int o = 16; o > 0; o >>= 1) s = __fadd_rn(s, __shfl_xor_sync(0xffffffffu, s, o));
-        if ((c & 31) == lane) {  // candidate c held by lane c % 32, slot c / 32
-            const int e = c >> 5;
+    for (int c0 = 0; c0 < kc; c0 += 4) {
+        uint32_t v[4];
+        float s[4];
 #pragma unroll
-            for (int q = 0; q < E; ++q)
-                if (q == e) keys[q] = ((uint64_t)f2ord(s) << 32) | v;
+        for (int q = 0; q < 4; ++q) {
+            v[q] = c0 + q < kc ? __ldg(cand + p * kc + c0 + q) : ANN_PAD;
+            s[q] = 0.0f;
+        }
+        for (int t = lane; t < d; t += 32) {
+            const float x = load_elem(Xrow, DT, u * d + t);
+#pragma unroll
+            for (int q = 0; q < 4; ++q) {
+                const float y = load_elem(X, DT, (int64_t)(v[q] == ANN_PAD ? 0 : v[q]) * d + t);
+                const float df = __fsub_rn(x, y);
+                s[q] = __fadd_rn(s[q], __fmul_rn(df, df));
+            }
+        }
+        for (int o = 16; o > 0; o >>= 1) {
+#pragma unroll
+            for (int q = 0; q < 4; ++q)
+                s[q] = __fadd_rn(s[q], __shfl_xor_sync(0xffffffffu, s[q], o));
+        }
+#pragma unroll
+        for (int q = 0; q < 4; ++q) {
+            const int c = c0 + q;
+            if ((c & 31) == lane && v[q] != ANN_PAD) {  // candidate c: lane c % 32, slot c / 32
+                const int e = c >> 5;
+#pragma unroll
+                for (int z = 0; z < E; ++z)
+                    if (z == e) keys[z] = ((uint64_t)f2ord(s[q]) << 32) | v[q];
+            }
         }
     }
     warp_bitonic_u64<E>(keys);
@@ -1837,12 +2017,8 @@ __global__ void k_rerank_vec(const void* X, const void* Xrow, int d,
             Chunk16<DT>::unpack(wa, fa);
             Chunk16<DT>::unpack(w0, f0);
             Chunk16<DT>::unpack(w1, f1);
-#pragma unroll
-            for (int t = 0; t < V; ++t) {
-                const float d0 = __fsub_rn(fa[t], f0[t]), d1 = __fsub_rn(fa[t], f1[t]);
-                s0 = __fadd_rn(s0, __fmul_rn(d0, d0));
-                s1 = __fadd_rn(s1, __fmul_rn(d1, d1));
-            }
+            s0 = sq_diff_add<V>(fa, f0, s0);
+            s1 = sq_diff_add<V>(fa, f1, s1);
         }
 #pragma unroll
         for (int o = 16; o > 0; o >>= 1) {
@@ -1919,11 +2095,7 @@ __global__ void k_rerank_g8(const void* X, const void* Xrow, int d,
             if (ch < nch) {
                 float f[V];
                 Chunk16<DT>::unpack(__ldg(xv + ch), f);
-#pragma unroll
-                for (int t = 0; t < V; ++t) {
-                    const float df = __fsub_rn(fa[q][t], f[t]);
-                    s = __fadd_rn(s, __fmul_rn(df, df));
-                }
+                s = sq_diff_add<V>(fa[q], f, s);
             }
         }
         s = __fadd_rn(s, __shfl_xor_sync(0xffffffffu, s, 4));
@@ -2780,23 +2952,22 @@ static int launch_rerank(const void* X, const void* Xrow, int dtype, int d, cons
 #define ANN_RERANK_VEC_W(DT)                                                                   \
     if (kc <= 64) ANN_RERANK_VEC(2, DT); else if (kc <= 128) ANN_RERANK_VEC(4, DT);              \
     else ANN_RERANK_VEC(8, DT);
-    if (vec) {
-        switch (dtype) {
-        case ANN_F32: ANN_RERANK_VEC_W(ANN_F32) break;
-        case ANN_F16: ANN_RERANK_VEC_W(ANN_F16) break;
-        case ANN_BF16: ANN_RERANK_VEC_W(ANN_BF16) break;
-        default: ANN_RERANK_VEC_W(ANN_U8) break;
-        }
-    } else if (kc <= 64) {
-        k_rerank<2><<<grid, threads, 0, st>>>(X, Xrow, dtype, d, row_ids, nwarps, cand, kc, k,
-                                              out_id, out_d, order);
-    } else if (kc <= 128) {
-        k_rerank<4><<<grid, threads, 0, st>>>(X, Xrow, dtype, d, row_ids, nwarps, cand, kc, k,
-                                              out_id, out_d, order);
-    } else {
-        k_rerank<8><<<grid, threads, 0, st>>>(X, Xrow, dtype, d, row_ids, nwarps, cand, kc, k,
-                                              out_id, out_d, order);
+#define ANN_RERANK(E, DT)                                                                      \
+    k_rerank<E, DT><<<grid, threads, 0, st>>>(X, Xrow, d, row_ids, nwarps, cand, kc, k, out_id, \
+                                              out_d, order)
+#define ANN_RERANK_W(DT)                                                                       \
+    if (vec) { ANN_RERANK_VEC_W(DT) }                                                          \
+    else if (kc <= 64) ANN_RERANK(2, DT);                                                      \
+    else if (kc <= 128) ANN_RERANK(4, DT);                                                     \
+    else ANN_RERANK(8, DT);
+    switch (dtype) {
+    case ANN_F32: ANN_RERANK_W(ANN_F32) break;
+    case ANN_F16: ANN_RERANK_W(ANN_F16) break;
+    case ANN_BF16: ANN_RERANK_W(ANN_BF16) break;
+    default: ANN_RERANK_W(ANN_U8) break;
     }
+#undef ANN_RERANK_W
+#undef ANN_RERANK
 #undef ANN_RERANK_VEC_W
 #undef ANN_RERANK_VEC
     ANN_CHECK_LAUNCH();
@@ -2985,7 +3156,7 @@ int run_shard_knn(const void* X, int64_t N, int d, int dtype, const uint32_t* me
     if ((rc = side_stream(&side, &fork_ev, &join_ev))) return rc;
     ANN_CHECK_CUDA(cudaEventRecord(fork_ev, st));
     ANN_CHECK_CUDA(cudaStreamWaitEvent(side, fork_ev, 0));
-    if ((rc = launch_pivot_chain(X, dtype, d, w, C, side))) return rc;
+    if ((rc = launch_pivot_chain(X, dtype, d, offsets, w, C, cell, side))) return rc;
     ANN_CHECK_CUDA(cudaEventRecord(join_ev, side));
     if ((rc = launch_gather(X, dtype, d, w.src, w.rows_cap, pl, w.G, w.norms, w.aug, amax, st)))
         return rc;
