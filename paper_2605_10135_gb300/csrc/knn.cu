@@ -166,6 +166,10 @@ struct KnnParams {
     // the sorted list of pool row p goes to split_list[p k' ...] as (order bits of the
     // key << 32 | id) instead of the outputs (NULL: no splits).
     uint64_t* split_list;
+    // Window mode (skipping bounds, see window_bound): where each row's and each row
+    // block's bound goes (NULL: the kNN sweep).
+    float* win_rowub;
+    float* win_bub;
     // Optional upper bound of every A row's k'-th squared distance (rowub[a]; NULL:
     // none): the sweep starts with that threshold.  Keys of split operands carry an
     // error, covered by the relative margin ub_margin (0 for exact keys); keys of
@@ -636,10 +640,68 @@ __device__ __forceinline__ int tile_at(int tt, int t0, int ntiles) {
     return right > left ? t0 + m + extra : t0 - m - extra;
 }
 
+// Window mode: an upper bound of every row's k'-th squared distance, from its tile
+// keys to the 256-row window that holds its block (two warps a row, 128 keys a thread in
+// registers).  An interpolating search on the key values, the counts of the two halves
+// added through shared memory in each step, keeps a value with at least k' keys at or
+// below it and stops within two of k': any such value is a bound.  +inf where the
+// window has fewer than k' other rows.  Both warps of a quarter compute the same
+// steps from the same sums, so they take the same barriers (also after an abort: then
+// a half's keys are +inf).
+__device__ __forceinline__ void pair_sync(int q) {
+    asm volatile("bar.sync %0, 64;" ::"r"(1 + q) : "memory");
+}
+__device__ __forceinline__ float window_bound(const float (&key)[128], int kp, int q, int h,
+                                              volatile float* ex /* [2][2][3][128] */) {
+    const int row = q * 32 + (threadIdx.x & 31);
+    float lo = INFINITY, hi = -INFINITY;
+    int n = 0;
+#pragma unroll
+    for (int u = 0; u < 128; ++u) {
+        const bool v = key[u] < INFINITY;
+        n += v ? 1 : 0;
+        lo = fminf(lo, key[u]);
+        hi = fmaxf(hi, v ? key[u] : -INFINITY);
+    }
+    auto slot = [&](int buf, int half, int f) { return ((buf * 2 + half) * 3 + f) * 128 + row; };
+    ex[slot(0, h, 0)] = (float)n;
+    ex[slot(0, h, 1)] = lo;
+    ex[slot(0, h, 2)] = hi;
+    pair_sync(q);
+    n += (int)ex[slot(0, 1 - h, 0)];
+    lo = fminf(lo, ex[slot(0, 1 - h, 1)]);
+    hi = fmaxf(hi, ex[slot(0, 1 - h, 2)]);
+    int clo = 0, chi = n;  // #{key <= hi} = chi, #{key < lo} = clo < kp
+    const bool none = n < kp;
+    for (int it = 1; it <= 14; ++it) {
+        const bool done = none || chi <= kp + 2 || !(lo < hi);
+        if (__all_sync(0xffffffffu, done)) break;
+        const float f = (it & 3) ? ((float)(kp + 1 - clo) / (float)(chi - clo)) : 0.5f;
+        float p = fmaf(f, hi - lo, lo);
+        p = p < hi ? p : 0.5f * lo + 0.5f * hi;
+        int c = 0;
+#pragma unroll
+        for (int u = 0; u < 128; ++u) c += key[u] <= p ? 1 : 0;
+        ex[slot(it & 1, h, 0)] = (float)c;
+        pair_sync(q);
+        c += (int)ex[slot(it & 1, 1 - h, 0)];
+        if (!done) {
+            if (c >= kp) {
+                hi = p;
+                chi = c;
+            } else {
+                lo = p;
+                clo = c;
+            }
+        }
+    }
+    return none ? INFINITY : hi;
+}
+
 // EMX: pool entries per row half / 32 that the compaction holds in registers
 // (ph <= 32 EMX); the common pools (ph <= 256) and the small ones (ph <= 96) use
 // instantiations of their own.
-template <int BN, bool PROF, int EMX>
+template <int BN, bool PROF, int EMX, bool WIN = false>
 __global__ void __launch_bounds__(kt::THREADS, 1)
     k_knn_tiles(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUtensorMap tmB,
                 const __grid_constant__ CUtensorMap tmAaug,
@@ -671,7 +733,12 @@ __global__ void __launch_bounds__(kt::THREADS, 1)
     const uint16_t* tlist =
         (P.tlist && ntiles <= kt::TL_MAX && P.tcount[bid] >= 0) ? P.tlist + bid * kt::TL_MAX
                                                                : nullptr;
-    const int nrun = tlist ? P.tcount[bid] : ntiles;
+    // Window mode: the tiles of the 256-row window that holds the block.
+    const int win0 = (rb >> 1) * (256 / BN);
+    const int nrun = WIN ? min(256 / BN, ntiles - win0) : tlist ? P.tcount[bid] : ntiles;
+    auto tile_of = [&](int run) {
+        return WIN ? win0 + run : tlist ? (int)tlist[run] : tile_at(run, t0, ntiles);
+    };
 
     uint8_t* base = (uint8_t*)(((uintptr_t)smem_raw + 1023) & ~(uintptr_t)1023);
     const KnnSmemLayout L = knn_smem_layout(BN, P.nkb_a, P.nst, P.a_stream);
@@ -733,7 +800,7 @@ __global__ void __launch_bounds__(kt::THREADS, 1)
                 if (d < INFINITY) t = 0.5f * __fsub_ru(d, nx);
             }
         }
-        ((uint32_t*)(base + L.tau))[row] = f2ord(t);
+        ((uint32_t*)(base + L.tau))[row] = WIN ? 0u : f2ord(t);
         ((float*)(base + L.tau))[kt::BM + row] = INFINITY;
         ((float*)(base + L.tau))[2 * kt::BM + row] = INFINITY;
     }
@@ -766,7 +833,7 @@ __global__ void __launch_bounds__(kt::THREADS, 1)
             bool ok = true;
             unsigned long long prod_wait = 0;
             for (int run = 0; run < nrun && ok;) {
-                const int t = tlist ? (int)tlist[run] : tile_at(run, t0, ntiles);
+                const int t = tile_of(run);
                 ++run;
                 const int b_y = (int)(pr.b_row0 + (int64_t)t * BN);
                 // the norm block first: its MMA opens the tile, so the slot frees early
@@ -957,9 +1024,63 @@ __global__ void __launch_bounds__(kt::THREADS, 1)
         // [128h, 128h + 128) of every tile.
         const int q = warp & 3;
         const int h = (warp - kt::EPI_WARP0) >> 2;
-        EpiState s;
         const int i = rb * kt::BM + q * 32 + lane;  // row index inside the problem
         const int i0 = rb * kt::BM + q * 32;        // first row of this warp
+        const uint32_t lane_addr = (uint32_t)(q * 32) << 16;
+        constexpr int HALF = BN / 2;
+        bool ok = true;
+        if constexpr (WIN) {
+            float key[128];
+#pragma unroll
+            for (int run = 0; run < 256 / BN; ++run) {
+                int there = run < nrun && ok ? 1 : 0;
+                if (there && lane == 0) there = mbar_wait(accf_bar + 8 * run, 0, abort_flag);
+                there = __shfl_sync(0xffffffffu, there, 0);
+                ok = ok && (there || run >= nrun);
+                tc_fence_after();
+                const int jt = (win0 + run) * BN + h * HALF;
+#pragma unroll
+                for (int c = 0; c < HALF / 32; ++c) {
+                    uint32_t v[32];
+                    if (there) {
+                        tmem_ld32(tmem + lane_addr + run * BN + h * HALF + c * 32, v);
+                        tmem_wait_ld32(v);
+                    }
+#pragma unroll
+                    for (int u = 0; u < 32; ++u) {
+                        const int j = jt + c * 32 + u;
+                        const bool col = there && j < pr.n_cols && j != i;
+                        key[run * HALF + c * 32 + u] = col ? __uint_as_float(v[u]) : INFINITY;
+                    }
+                }
+            }
+            const float kb = window_bound(key, P.kprime, q, h, (volatile float*)(base + L.kscr));
+            float ub = INFINITY;
+            if (i < pr.n_rows && kb < INFINITY) {
+                // |x - y|^2 = |x|^2 + 2 key, rounded up, and the error of inexact keys (an
+                // eighth of ub_margin times |x|^2 + |y|^2 <= 3 |x|^2 + 2 dist); the scale of
+                // scaled operands is a power of two
+                const float nx = P.na[pr.a_row0 + i];
+                ub = fmaxf(__fmaf_ru(2.0f, kb, nx), 0.0f);
+                ub = __fmaf_ru(0.125f * P.ub_margin, __fmaf_ru(3.0f, nx, 2.0f * ub), ub);
+                if (P.ub_amax) {
+                    const float inv = 1.0f / operand_scale(*P.ub_amax, false);
+                    ub = __fmul_ru(__fmul_ru(ub, inv), inv);
+                }
+                if (!(ub >= 0.0f)) ub = INFINITY;
+            }
+            if (h == 0) {
+                if (i < pr.n_rows) P.win_rowub[pr.a_row0 + i] = ub;
+                const uint32_t m = __reduce_max_sync(
+                    0xffffffffu, i < pr.n_rows ? __float_as_uint(ub) : 0u);
+                if (lane == 0) atomicMax((uint32_t*)(base + L.tau), m);
+            }
+            if (!ok) {
+                *abort_flag = 1;
+                if (lane == 0) atomicOr(P.status, DEV_TIMEOUT);
+            }
+        } else {
+        EpiState s;
         s.ph = P.ph;
         s.c = 0;
         s.kp = P.kprime;
@@ -977,11 +1098,8 @@ __global__ void __launch_bounds__(kt::THREADS, 1)
         unsigned long long e_wait = 0;
         long long e_t0 = 0;
         if (PROF) e_t0 = clock64();
-        const uint32_t lane_addr = (uint32_t)(q * 32) << 16;
-        bool ok = true;
-        constexpr int HALF = BN / 2;
         for (int run = 0; run < nrun;) {
-            const int t = tlist ? (int)tlist[run] : tile_at(run, t0, ntiles);
+            const int t = tile_of(run);
             const int a = run % kt::NACC;
             const int par = (run / kt::NACC) & 1;
             ++run;
@@ -1060,9 +1178,11 @@ __global__ void __launch_bounds__(kt::THREADS, 1)
             else
                 P.pool_cnt[(pr.pool_row0 + i) * 2 + h] = ok ? s.c : 0;
         }
+        }
     }
     tc_fence_before();
     __syncthreads();
+    if (WIN && threadIdx.x == 0) P.win_bub[bid] = __uint_as_float(*(const uint32_t*)(base + L.tau));
     if (PROF && threadIdx.x == 0) {
         prof_add(TC_CTA_CYCLES, (unsigned long long)(clock64() - cta_t0));
         prof_add(TC_CTAS, 1);
@@ -2292,7 +2412,10 @@ static inline size_t row_bytes(const KnnPlan& pl) { return (size_t)pl.Kp * (pl.e
 // the same shard), with centres c_A, c_G and radii r_A >= max |x - c_A|, r_G, every
 // pair satisfies |x - y| >= |c_A - c_G| - r_A - r_G (triangle inequality).  The k-th
 // distance of each row among the other rows of its 256-row window bounds its final
-// k-th squared distance from above (k_ub_own); a column tile whose
+// k-th squared distance from above (the window mode of the tile kernel: one tile a row
+// block on the tensor cores and a search of its keys; direct distances with dp4a or
+// 8 x 8 FP32 register tiles took 5.2 ms for 2M uint8 rows of 128 and 84 ms for 20M FP32
+// rows of 96, this 1.3 and 13.5 ms); a column tile whose
 // groups all lie beyond the block's largest bound cannot hold a neighbour of any of
 // its rows, so the sweep skips it (its copies, products and epilogue).  Ties stay
 // exact: a skipped column is strictly farther than the bound.  Used for plain
@@ -2389,198 +2512,6 @@ __device__ __forceinline__ int block_problem(const int64_t* __restrict__ blk_off
         if (blk_off[mid] <= bid) lo = mid; else hi = mid - 1;
     }
     return lo;
-}
-
-// bub[bid] = the largest, over the block's rows, k-th smallest squared distance
-// from the row to the other valid rows of its 256-row window of the shard (the
-// window holding the block), or +inf where a row has fewer than k others there:
-// an upper bound of every row's final k-th distance.  uint8 vectors with d a
-// multiple of 4, NW4 = d / 4 words at most; exact integer arithmetic
-// (|x|^2 + |y|^2 - 2 x.y with dp4a).  One block of 256 threads per row block; the
-// window's vectors are staged in shared memory, each row's words held in registers.
-template <int NW4>
-__global__ void __launch_bounds__(256)
-k_ub_own(const uint8_t* __restrict__ X, int d, const int64_t* __restrict__ src,
-         const int64_t* __restrict__ blk_off, const KnnProblem* __restrict__ probs, int nprob,
-         int k, int64_t nblocks, float* __restrict__ bub, float* __restrict__ rowub) {
-    extern __shared__ uint32_t wv[];  // [256][ws] packed vectors, then [256] norms
-    __shared__ unsigned int bmax;
-    const int64_t bid = blockIdx.x;
-    if (bid >= nblocks) return;
-    if (bid >= blk_off[nprob]) {
-        if (threadIdx.x == 0) bub[bid] = INFINITY;
-        return;
-    }
-    const int p = block_problem(blk_off, nprob, bid);
-    const KnnProblem pr = probs[p];
-    const int rb = (int)(bid - blk_off[p]);
-    const int nw4 = d / 4;
-    const int ws = nw4 + 1;  // padded row stride (words): no bank conflicts across lanes
-    uint32_t* nrm = wv + 256 * ws;
-    const int c0 = (rb >> 1) * 256;  // first column of the window (shard-relative)
-    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-    if (tid == 0) bmax = 0;
-    // stage: warp w loads columns w, w + 8, ...; lane q loads word q (coalesced)
-    for (int c = warp; c < 256; c += 8) {
-        const bool valid = c0 + c < pr.n_cols;
-        const int64_t v = valid ? src[pr.b_row0 + c0 + c] : -1;
-        uint32_t n2 = 0;
-        for (int q = lane; q < nw4; q += 32) {
-            const uint32_t word = v >= 0 ? ((const uint32_t*)(X + v * d))[q] : 0u;
-            wv[c * ws + q] = word;
-            n2 = __dp4a(word, word, n2);
-        }
-        for (int o = 16; o; o >>= 1) n2 += __shfl_xor_sync(0xffffffffu, n2, o);
-        if (lane == 0) nrm[c] = v >= 0 ? n2 : 0xFFFFFFFFu;  // all ones: not a column
-    }
-    __syncthreads();
-    unsigned int wmax = 0;
-    for (int r = warp; r < kt::BM; r += 8) {
-        const int i = rb * kt::BM + r;  // row index in the shard
-        if (i >= pr.n_rows) continue;
-        const int cr = i - c0;          // the row's own column in the window
-        const uint32_t nr = nrm[cr];
-        uint32_t rw[NW4];
-#pragma unroll
-        for (int w = 0; w < NW4; ++w) rw[w] = w < nw4 ? wv[cr * ws + w] : 0u;
-        uint32_t dv[8];
-#pragma unroll
-        for (int q = 0; q < 8; ++q) {
-            const int c = lane + 32 * q;
-            const uint32_t nc = nrm[c];
-            const uint32_t* cw = wv + c * ws;
-            uint32_t dot = 0;
-#pragma unroll
-            for (int w = 0; w < NW4; ++w)
-                if (w < nw4) dot = __dp4a(rw[w], cw[w], dot);
-            dv[q] = (nc == 0xFFFFFFFFu || c == cr) ? 0xFFFFFFFFu : nr + nc - 2u * dot;
-        }
-        // k-th smallest of the window's distances: least v with #{dist <= v} >= k
-        int cnt = 0;
-#pragma unroll
-        for (int q = 0; q < 8; ++q) cnt += dv[q] != 0xFFFFFFFFu;
-        for (int o = 16; o; o >>= 1) cnt += __shfl_xor_sync(0xffffffffu, cnt, o);
-        unsigned int ub = 0xFFFFFFFFu;
-        if (cnt >= k) {
-            unsigned int lo = 0, hi = 1u << 24;  // squared distances of uint8 rows, d <= 256
-            while (lo < hi) {
-                const unsigned int mid = lo + (hi - lo) / 2;
-                int c = 0;
-#pragma unroll
-                for (int q = 0; q < 8; ++q) c += dv[q] <= mid;
-                for (int o = 16; o; o >>= 1) c += __shfl_xor_sync(0xffffffffu, c, o);
-                if (c >= k) hi = mid; else lo = mid + 1;
-            }
-            ub = lo;
-        }
-        if (rowub && lane == 0) rowub[pr.a_row0 + i] = ub == 0xFFFFFFFFu ? INFINITY : (float)ub;
-        wmax = ub > wmax ? ub : wmax;
-    }
-    if (lane == 0) atomicMax(&bmax, wmax);
-    __syncthreads();
-    if (tid == 0) bub[bid] = bmax == 0xFFFFFFFFu ? INFINITY : (float)bmax;
-}
-
-// As k_ub_own for float vectors (d <= 200): FP32 direct-form squared distances
-// (x - y)^2 summed in index order, the k-th smallest found by a search on the bit
-// patterns of the non-negative floats.  Register tiles: a warp takes 8 rows at a
-// time and each lane 8 window columns (lane + 32 q), so one pass over the
-// dimensions reads 8 broadcast row values and 8 column values from shared memory
-// for 64 products.
-__global__ void __launch_bounds__(256)
-k_ub_own_f32(const float* __restrict__ X, int d, const int64_t* __restrict__ src,
-             const int64_t* __restrict__ blk_off, const KnnProblem* __restrict__ probs, int nprob,
-             int k, int64_t nblocks, float* __restrict__ bub, float* __restrict__ rowub) {
-    extern __shared__ float wf[];  // [256][d + 1]
-    __shared__ unsigned int bmax;
-    const int64_t bid = blockIdx.x;
-    if (bid >= nblocks) return;
-    if (bid >= blk_off[nprob]) {
-        if (threadIdx.x == 0) bub[bid] = INFINITY;
-        return;
-    }
-    const int p = block_problem(blk_off, nprob, bid);
-    const KnnProblem pr = probs[p];
-    const int rb = (int)(bid - blk_off[p]);
-    const int ws = d + 1;
-    const int c0 = (rb >> 1) * 256;
-    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-    __shared__ unsigned char cvalid[256];
-    if (tid == 0) bmax = 0;
-    for (int c = warp; c < 256; c += 8) {
-        const bool valid = c0 + c < pr.n_cols;
-        const int64_t v = valid ? src[pr.b_row0 + c0 + c] : -1;
-        for (int t = lane; t < d; t += 32) wf[c * ws + t] = v >= 0 ? X[v * d + t] : 0.0f;
-        if (lane == 0) cvalid[c] = v >= 0;
-    }
-    __syncthreads();
-    const uint32_t NONE = 0x7F800000u;  // +inf: not a column
-    unsigned int wmax = 0;
-    for (int g = 0; g < 2; ++g) {
-        const int r0 = warp * 16 + g * 8;  // rows r0 .. r0 + 7 of the block
-        const int i0 = rb * kt::BM + r0;   // their row index in the shard
-        if (i0 >= pr.n_rows) break;
-        float acc[8][8];
-#pragma unroll
-        for (int j = 0; j < 8; ++j)
-#pragma unroll
-            for (int q = 0; q < 8; ++q) acc[j][q] = 0.0f;
-        const float* xr = wf + (i0 - c0) * ws;  // row r0's own window column
-        const float* xc = wf + lane * ws;
-        for (int t = 0; t < d; ++t) {
-            float a[8], b[8];
-#pragma unroll
-            for (int j = 0; j < 8; ++j) a[j] = xr[j * ws + t];
-#pragma unroll
-            for (int q = 0; q < 8; ++q) b[q] = xc[32 * q * ws + t];
-#pragma unroll
-            for (int j = 0; j < 8; ++j)
-#pragma unroll
-                for (int q = 0; q < 8; ++q) {
-                    const float df = a[j] - b[q];
-                    acc[j][q] = fmaf(df, df, acc[j][q]);
-                }
-        }
-#pragma unroll
-        for (int j = 0; j < 8; ++j) {
-            const int i = i0 + j;
-            if (i >= pr.n_rows) break;  // warp-uniform
-            const int cr = i - c0;       // the row's own column in the window
-            uint32_t dv[8];
-            int cnt = 0;
-#pragma unroll
-            for (int q = 0; q < 8; ++q) {
-                const int c = lane + 32 * q;
-                dv[q] = (!cvalid[c] || c == cr) ? NONE : __float_as_uint(acc[j][q]);
-                cnt += dv[q] != NONE;
-            }
-            cnt = __reduce_add_sync(0xffffffffu, cnt);
-            unsigned int ub = NONE;
-            if (cnt >= k) {
-                unsigned int lo = 0, hi = NONE;
-                while (lo < hi) {
-                    const unsigned int mid = lo + (hi - lo) / 2;
-                    unsigned int c = 0;
-#pragma unroll
-                    for (int q = 0; q < 8; ++q) c += dv[q] <= mid;
-                    c = __reduce_add_sync(0xffffffffu, c);
-                    if (c >= (unsigned int)k) hi = mid; else lo = mid + 1;
-                }
-                ub = lo;
-            }
-            // FP32 sums of d squares: relative error below (d + 2) 2^-24; pushed up
-            if (rowub && lane == 0)
-                rowub[pr.a_row0 + i] =
-                    ub >= NONE ? INFINITY : __uint_as_float(ub) * (1.0f + (float)(d + 4) * 0x1p-22f);
-            wmax = ub > wmax ? ub : wmax;
-        }
-    }
-    if (lane == 0) atomicMax(&bmax, wmax);
-    __syncthreads();
-    // FP32 sums of d squares: relative error below (d + 2) 2^-24; pushed up
-    if (tid == 0)
-        bub[bid] = bmax >= NONE ? INFINITY
-                                : __uint_as_float(bmax) * (1.0f + (float)(d + 4) * 0x1p-22f);
 }
 
 // tlist[bid]: the column tiles a row block sweeps, nearest first.  A tile is left
@@ -2861,6 +2792,15 @@ static int launch_tiles(const KnnPlan& pl, const void* GA, int64_t rowsA, const 
     if (!rc)
         rc = make_tmap(&tba, augB, rowsB, kt::KAUG, kt::KAUG, pl.bn, CU_TENSOR_MAP_SWIZZLE_32B);
     if (rc) return rc;
+    if (P.win_rowub) {
+        auto kern = pl.bn == 256 ? k_knn_tiles<256, false, 8, true> : k_knn_tiles<128, false, 8, true>;
+        ANN_CHECK_CUDA(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                            (int)pl.smem));
+        if (grid <= 0) return ANN_OK;
+        kern<<<(unsigned)grid, kt::THREADS, pl.smem, st>>>(ta, tb, taa, tba, P);
+        ANN_CHECK_LAUNCH();
+        return ANN_OK;
+    }
     const bool prof = timed && tile_counters_on();
     constexpr int EBIG = kt::PH_MAX / 32;
     const bool big = P.ph > 256, small = P.ph <= 96;
@@ -3013,6 +2953,8 @@ static KnnParams base_params(const KnnPlan& pl, int k, const int64_t* blk_off,
     P.ub_margin = 0.0f;
     P.ub_amax = nullptr;
     P.split_list = nullptr;
+    P.win_rowub = nullptr;
+    P.win_bub = nullptr;
     return P;
 }
 
@@ -3207,20 +3149,7 @@ int run_shard_knn(const void* X, int64_t N, int d, int dtype, const uint32_t* me
             X, dtype, d, w.src, ng, pl.Kp, w.gcent, w.grad, w.gmaxn);
         ANN_CHECK_LAUNCH();
         float kslack = 0.0f;
-        if (skip_u8) {
-            const size_t ubs = ((size_t)256 * (d / 4 + 1) + 256) * sizeof(uint32_t);
-            if (d <= 128) {
-                ANN_CHECK_CUDA(cudaFuncSetAttribute(
-                    k_ub_own<32>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)ubs));
-                k_ub_own<32><<<(unsigned)grid, 256, ubs, st>>>(
-                    (const uint8_t*)X, d, w.src, w.blk_off, w.probs, C, pl.kprime, grid, w.bub, w.rowub);
-            } else {
-                ANN_CHECK_CUDA(cudaFuncSetAttribute(
-                    k_ub_own<64>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)ubs));
-                k_ub_own<64><<<(unsigned)grid, 256, ubs, st>>>(
-                    (const uint8_t*)X, d, w.src, w.blk_off, w.probs, C, pl.kprime, grid, w.bub, w.rowub);
-            }
-        } else {
+        if (!skip_u8) {
             // Split BF16 keys (three products, FP32 accumulation): the error of a
             // squared distance stays below (2^-16 + (d + 4) 2^-24)(|x|^2 + |y|^2);
             // BF16 operands (each rounded once, relative 2^-9; the norms in FP32):
@@ -3231,13 +3160,14 @@ int run_shard_knn(const void* X, int64_t N, int d, int dtype, const uint32_t* me
             kslack = split_keys  ? 8.0f * (0x1p-16f + (float)(d + 4) * 0x1p-24f)
                      : bf16_keys ? 8.0f * (0x1p-8f + (float)(d + 8) * 0x1p-24f)
                                  : 8.0f * (0x1p-10f + (float)(d + 8) * 0x1p-24f);
-            const size_t ubs = (size_t)256 * (d + 1) * sizeof(float);
-            ANN_CHECK_CUDA(cudaFuncSetAttribute(
-                k_ub_own_f32, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)ubs));
-            k_ub_own_f32<<<(unsigned)grid, 256, ubs, st>>>(
-                (const float*)X, d, w.src, w.blk_off, w.probs, C, pl.kprime, grid, w.bub, w.rowub);
         }
-        ANN_CHECK_LAUNCH();
+        KnnParams W = P;
+        W.win_rowub = w.rowub;
+        W.win_bub = w.bub;
+        W.ub_margin = kslack;
+        W.ub_amax = pl.scaled ? amax : nullptr;
+        rc = launch_tiles(pl, w.G, w.rows_cap, w.ones, w.G, w.aug, w.rows_cap, W, grid, st, false);
+        if (rc) return rc;
         const size_t tls = tile_list_smem(d).total;
         ANN_CHECK_CUDA(cudaFuncSetAttribute(k_tile_list, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                             (int)tls));
