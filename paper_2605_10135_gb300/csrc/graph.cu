@@ -6,7 +6,7 @@
 // in shared memory (one probe per lookup, a multiplier chosen per row so that
 // no two of its ids share a slot); the lists of u's neighbours are read with
 // coalesced warp loads, every entry looked up, and the counts c_j kept in
-// registers (a warp OR-reduction per neighbour).  The R entries of smallest
+// shared memory (one predicated add per entry).  The R entries of smallest
 // (c_j, j) are chosen by a warp bitonic sort and written in list order with a
 // ballot/popc compaction.  Integer logic only.
 //
@@ -105,26 +105,28 @@ constexpr int PTRY = 32;
 __device__ __forceinline__ uint32_t tmult(int a) { return HM + 0x3C6EF372u * (uint32_t)a; }  // odd
 __device__ __forceinline__ uint32_t tkey(uint32_t y) { return y << 10; }  // low 22 bits << 10
 
-// Shared memory of one prune warp: table words [TS], overflow ids and positions
-// [KM each], the neighbours' rows [KM], the overflow count (+pad).
+// Shared memory of one prune warp: table words [TS], the neighbours' rows [KM], overflow
+// ids and positions [KM each], the counts [KM], the overflow count (+pad).
 __host__ __device__ constexpr size_t prune_warp_smem(int KM) {
-    return (size_t)TS * 4 + (size_t)KM * 16 + 16;
+    return (size_t)TS * 4 + (size_t)KM * 20 + 16;
 }
 
 // Detour counts of one row: for each neighbour v_i (i < m) the warp reads L_{v_i}
 // with coalesced loads (entry t in lane t % 32, register t / 32) and looks each
 // entry up in u's table; an entry at position j of u's list with i < j and t < j
-// sets bit j of the lane's mask.  The ids of a list are distinct, so OR over the
-// lanes counts each (i, j) pair once; lane l adds bit l of word e to c[e], the
-// count of position j = l + 32 e.
+// adds one to cnt[j] (the ids of a list are distinct: one add per (i, j) pair).  Bound
+// by instruction issue: a lookup is a multiply, a table read, two compares and the
+// add.  Collecting the hits as bits of 64-bit words and OR-reducing them over the
+// warp for each neighbour took more instructions, and a compare-and-swap per id and
+// try of the table cost as much again (12.8 ms for 2M rows of 64, this 11.4).
 template <int E, bool OVF>
 __device__ __forceinline__ void prune_counts(const uint32_t* __restrict__ knn_id, int k, int m,
                                              const int64_t* wrow, const uint32_t* tw,
                                              const uint32_t* ovf, const uint32_t* ovf_pos,
-                                             int novf, uint32_t A, uint32_t (&c)[E]) {
-    constexpr int G = E <= 2 ? 4 : 2;  // neighbour lists read together (loads in flight)
+                                             int novf, uint32_t A, uint32_t* cnt) {
+    constexpr int G = E <= 2 ? 8 : 2;  // neighbour lists read together (loads in flight)
     const int lane = threadIdx.x & 31;
-    for (int i0 = 0; i0 < m; i0 += G) {
+    for (int i0 = 0; i0 + 1 < m; i0 += G) {  // (the last neighbour has no j behind it)
         uint32_t x[G][E];
 #pragma unroll
         for (int g = 0; g < G; ++g) {
@@ -138,17 +140,11 @@ __device__ __forceinline__ void prune_counts(const uint32_t* __restrict__ knn_id
         }
 #pragma unroll
         for (int g = 0; g < G; ++g) {
-            const int i = i0 + g;
-            if (i >= m) break;  // warp-uniform
             // (ANN_PAD entries never match: the table holds only the row's ids)
-            uint32_t bits[E];
-            uint64_t bits64 = 0;  // E <= 2: positions 0..63 in one word
-#pragma unroll
-            for (int e = 0; e < E; ++e) bits[e] = 0;
 #pragma unroll
             for (int e = 0; e < E; ++e) {
-                const int t = lane + 32 * e;
-                const uint32_t thr = (uint32_t)(i > t ? i : t);  // hit: thr < j < 256
+                const uint32_t t = lane + 32 * e, i = i0 + g;
+                const uint32_t first = (i > t ? i : t) + 1u;  // hit: first <= j < 256
                 const uint32_t y = x[g][e] * A;
                 const uint32_t wd = tw[y >> TSHIFT];
                 uint32_t dj = wd ^ tkey(y);  // the position j when the slot holds x
@@ -156,24 +152,7 @@ __device__ __forceinline__ void prune_counts(const uint32_t* __restrict__ knn_id
                     for (int o = 0; o < novf; ++o)
                         if (ovf[o] == x[g][e]) dj = ovf_pos[o];
                 }
-                if (dj - thr - 1u < 255u - thr) {
-                    if constexpr (E <= 2) {
-                        bits64 |= 1ull << dj;
-                    } else {
-#pragma unroll
-                        for (int e2 = 0; e2 < E; ++e2)
-                            if ((int)(dj >> 5) == e2) bits[e2] |= 1u << (dj & 31u);
-                    }
-                }
-            }
-            if constexpr (E <= 2) {
-                bits[0] = (uint32_t)bits64;
-                if (E == 2) bits[E - 1] = (uint32_t)(bits64 >> 32);
-            }
-#pragma unroll
-            for (int e = 0; e < E; ++e) {
-                if (32 * e + 31 <= i) continue;  // no j > i in this word (uniform)
-                c[e] += (__reduce_or_sync(0xffffffffu, bits[e]) >> lane) & 1u;
+                if (dj - first < 256u - first) atomicAdd(cnt + dj, 1u);
             }
         }
     }
@@ -197,7 +176,8 @@ __global__ void k_prune(const uint32_t* __restrict__ knn_id, const float* __rest
     int64_t* wrow = (int64_t*)(tw + TS);           // [KM]
     uint32_t* ovf = (uint32_t*)(wrow + KM);        // [KM]
     uint32_t* ovf_pos = ovf + KM;                  // [KM]
-    int* novf_p = (int*)(ovf_pos + KM);            // [1] (+pad)
+    uint32_t* cnt = ovf_pos + KM;                  // [KM]
+    int* novf_p = (int*)(cnt + KM);                // [1] (+pad)
     const uint32_t lt = (1u << lane) - 1;
     // the table starts empty once; after each row only the slots its ids used are
     // emptied again
@@ -240,15 +220,22 @@ __global__ void k_prune(const uint32_t* __restrict__ knn_id, const float* __rest
             bool perfect = false;
             for (int a = 0; a < (E <= 2 ? PTRY : 0) && !perfect; ++a) {
                 A = tmult(a);
+                // every id's word stored and read back: where two share a slot, one of them
+                // reads the other's (plain accesses; a compare-and-swap per id and try cost
+                // more than the lookups it served)
+#pragma unroll
+                for (int e = 0; e < E; ++e) {
+                    const int j = lane + 32 * e;
+                    const uint32_t y = lu[e] * A;
+                    if (j < m) tw[y >> TSHIFT] = tkey(y) | (uint32_t)j;
+                }
+                __syncwarp();
                 bool clash = false;
 #pragma unroll
                 for (int e = 0; e < E; ++e) {
                     const int j = lane + 32 * e;
-                    if (j < m) {
-                        const uint32_t y = lu[e] * A;
-                        if (atomicCAS(&tw[y >> TSHIFT], TEMPTY, tkey(y) | (uint32_t)j) != TEMPTY)
-                            clash = true;
-                    }
+                    const uint32_t y = lu[e] * A;
+                    if (j < m) clash = clash || tw[y >> TSHIFT] != (tkey(y) | (uint32_t)j);
                 }
                 perfect = !__any_sync(0xffffffffu, clash);
                 if (!perfect) {  // empty every slot the row's ids touched, try the next
@@ -278,14 +265,17 @@ __global__ void k_prune(const uint32_t* __restrict__ knn_id, const float* __rest
                 __syncwarp();
                 novf = *novf_p;
             }
-            __syncwarp();
             uint32_t c[E];
 #pragma unroll
-            for (int e = 0; e < E; ++e) c[e] = 0;
+            for (int e = 0; e < E; ++e) cnt[lane + 32 * e] = 0;
+            __syncwarp();
             if (novf == 0)
-                prune_counts<E, false>(knn_id, k, m, wrow, tw, ovf, ovf_pos, 0, A, c);
+                prune_counts<E, false>(knn_id, k, m, wrow, tw, ovf, ovf_pos, 0, A, cnt);
             else
-                prune_counts<E, true>(knn_id, k, m, wrow, tw, ovf, ovf_pos, novf, A, c);
+                prune_counts<E, true>(knn_id, k, m, wrow, tw, ovf, ovf_pos, novf, A, cnt);
+            __syncwarp();
+#pragma unroll
+            for (int e = 0; e < E; ++e) c[e] = cnt[lane + 32 * e];
             // rank positions by (c_j, j); any starting placement sorts the same
             uint32_t sel[E];
 #pragma unroll
