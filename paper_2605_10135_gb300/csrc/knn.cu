@@ -647,29 +647,56 @@ __device__ __forceinline__ int tile_at(int tt, int t0, int ntiles) {
     return right > left ? t0 + m + extra : t0 - m - extra;
 }
 
-// Window mode: an upper bound of every row's k'-th squared distance, from its tile
-// keys to the 256-row window that holds its block (two warps a row, 128 keys a thread in
-// registers).  An interpolating search on the key values, the counts of the two halves
-// added through shared memory in each step, keeps a value with at least k' keys at or
-// below it and stops within two of k': any such value is a bound.  +inf where the
-// window has fewer than k' other rows.  Both warps of a quarter compute the same
-// steps from the same sums, so they take the same barriers (also after an abort: then
-// a half's keys are +inf).
+// Window mode: an upper bound of every row's k'-th squared distance, from its tile keys
+// to the two tiles (512 columns, 256 with narrow tiles) that hold its block, kept in
+// TMEM: two warps a row, each reading its half of the columns anew in every step.  An
+// interpolating search on the key values, the counts of the two halves added through
+// shared memory in each step, keeps a value with at least k' keys at or below it and
+// stops within two of k': any such value is a bound.  +inf where the window has fewer
+// than k' other rows.  Both warps of a quarter compute the same steps from the same
+// sums, so they take the same barriers (also after an abort: then a half has no keys).
+// The wider the window, the nearer its k'-th key is to the row's: with 256 columns and
+// keys in registers 256-wide lists had no bound at all.
 __device__ __forceinline__ void pair_sync(int q) {
     asm volatile("bar.sync %0, 64;" ::"r"(1 + q) : "memory");
 }
-__device__ __forceinline__ float window_bound(const float (&key)[128], int kp, int q, int h,
+// f(key) of every key of the thread's row and half: runs tiles of BN columns at tb,
+// columns j0 + run BN ...; columns from n_cols on and the row's own are skipped.
+template <int BN, class F>
+__device__ __forceinline__ void window_keys(uint32_t tb, int runs, int j0, int i, int n_cols, F f) {
+    const int i0 = i - (int)(threadIdx.x & 31);
+    for (int run = 0; run < runs; ++run) {
+#pragma unroll 1
+        for (int c = 0; c < BN / 2; c += 32) {
+            uint32_t v[32];
+            __syncwarp();
+            tmem_ld32(tb + run * BN + c, v);
+            tmem_wait_ld32(v);
+            const int j = j0 + run * BN + c;
+            if (j + 32 > n_cols || (i0 + 32 > j && i0 < j + 32)) {  // warp-uniform
+#pragma unroll
+                for (int u = 0; u < 32; ++u)
+                    if (j + u < n_cols && j + u != i) f(__uint_as_float(v[u]));
+            } else {
+#pragma unroll
+                for (int u = 0; u < 32; ++u) f(__uint_as_float(v[u]));
+            }
+        }
+    }
+}
+template <int BN>
+__device__ __forceinline__ float window_bound(uint32_t tb, int runs, int j0, int i, int n_cols,
+                                              int kp, int q, int h,
                                               volatile float* ex /* [2][2][3][128] */) {
     const int row = q * 32 + (threadIdx.x & 31);
     float lo = INFINITY, hi = -INFINITY;
     int n = 0;
-#pragma unroll
-    for (int u = 0; u < 128; ++u) {
-        const bool v = key[u] < INFINITY;
+    window_keys<BN>(tb, runs, j0, i, n_cols, [&](float x) {
+        const bool v = x < INFINITY;
         n += v ? 1 : 0;
-        lo = fminf(lo, key[u]);
-        hi = fmaxf(hi, v ? key[u] : -INFINITY);
-    }
+        lo = fminf(lo, x);
+        hi = fmaxf(hi, v ? x : -INFINITY);
+    });
     auto slot = [&](int buf, int half, int f) { return ((buf * 2 + half) * 3 + f) * 128 + row; };
     ex[slot(0, h, 0)] = (float)n;
     ex[slot(0, h, 1)] = lo;
@@ -687,8 +714,7 @@ __device__ __forceinline__ float window_bound(const float (&key)[128], int kp, i
         float p = fmaf(f, hi - lo, lo);
         p = p < hi ? p : 0.5f * lo + 0.5f * hi;
         int c = 0;
-#pragma unroll
-        for (int u = 0; u < 128; ++u) c += key[u] <= p ? 1 : 0;
+        window_keys<BN>(tb, runs, j0, i, n_cols, [&](float x) { c += x <= p ? 1 : 0; });
         ex[slot(it & 1, h, 0)] = (float)c;
         pair_sync(q);
         c += (int)ex[slot(it & 1, 1 - h, 0)];
@@ -740,9 +766,9 @@ __global__ void __launch_bounds__(kt::THREADS, 1)
     const uint16_t* tlist =
         (P.tlist && ntiles <= kt::TL_MAX && P.tcount[bid] >= 0) ? P.tlist + bid * kt::TL_MAX
                                                                : nullptr;
-    // Window mode: the tiles of the 256-row window that holds the block.
-    const int win0 = (rb >> 1) * (256 / BN);
-    const int nrun = WIN ? min(256 / BN, ntiles - win0) : tlist ? P.tcount[bid] : ntiles;
+    // Window mode: the two tiles that hold the block (their accumulators stay in TMEM).
+    const int win0 = rb * kt::BM / (2 * BN) * 2;
+    const int nrun = WIN ? min(2, ntiles - win0) : tlist ? P.tcount[bid] : ntiles;
     auto tile_of = [&](int run) {
         return WIN ? win0 + run : tlist ? (int)tlist[run] : tile_at(run, t0, ntiles);
     };
@@ -1037,31 +1063,15 @@ __global__ void __launch_bounds__(kt::THREADS, 1)
         constexpr int HALF = BN / 2;
         bool ok = true;
         if constexpr (WIN) {
-            float key[128];
-#pragma unroll
-            for (int run = 0; run < 256 / BN; ++run) {
-                int there = run < nrun && ok ? 1 : 0;
-                if (there && lane == 0) there = mbar_wait(accf_bar + 8 * run, 0, abort_flag);
-                there = __shfl_sync(0xffffffffu, there, 0);
-                ok = ok && (there || run >= nrun);
-                tc_fence_after();
-                const int jt = (win0 + run) * BN + h * HALF;
-#pragma unroll
-                for (int c = 0; c < HALF / 32; ++c) {
-                    uint32_t v[32];
-                    if (there) {
-                        tmem_ld32(tmem + lane_addr + run * BN + h * HALF + c * 32, v);
-                        tmem_wait_ld32(v);
-                    }
-#pragma unroll
-                    for (int u = 0; u < 32; ++u) {
-                        const int j = jt + c * 32 + u;
-                        const bool col = there && j < pr.n_cols && j != i;
-                        key[run * HALF + c * 32 + u] = col ? __uint_as_float(v[u]) : INFINITY;
-                    }
-                }
+            for (int run = 0; run < nrun && ok; ++run) {
+                int there = 1;
+                if (lane == 0) there = mbar_wait(accf_bar + 8 * run, 0, abort_flag);
+                ok = __shfl_sync(0xffffffffu, there, 0) != 0;
             }
-            const float kb = window_bound(key, P.kprime, q, h, (volatile float*)(base + L.kscr));
+            tc_fence_after();
+            const float kb = window_bound<BN>(tmem + lane_addr + h * HALF, ok ? nrun : 0,
+                                              win0 * BN + h * HALF, i, pr.n_cols, P.kprime, q, h,
+                                              (volatile float*)(base + L.kscr));
             float ub = INFINITY;
             if (i < pr.n_rows && kb < INFINITY) {
                 // |x - y|^2 = |x|^2 + 2 key, rounded up, and the error of inexact keys (an
@@ -2418,11 +2428,11 @@ static inline size_t row_bytes(const KnnPlan& pl) { return (size_t)pl.Kp * (pl.e
 // For a row block A (128 gathered rows) and a column group G (128 gathered rows of
 // the same shard), with centres c_A, c_G and radii r_A >= max |x - c_A|, r_G, every
 // pair satisfies |x - y| >= |c_A - c_G| - r_A - r_G (triangle inequality).  The k-th
-// distance of each row among the other rows of its 256-row window bounds its final
+// distance of each row among the other rows of its 512-row window bounds its final
 // k-th squared distance from above (the window mode of the tile kernel: one tile a row
 // block on the tensor cores and a search of its keys; direct distances with dp4a or
 // 8 x 8 FP32 register tiles took 5.2 ms for 2M uint8 rows of 128 and 84 ms for 20M FP32
-// rows of 96, this 1.3 and 13.5 ms); a column tile whose
+// rows of 96, this about 2 and 18 ms); a column tile whose
 // groups all lie beyond the block's largest bound cannot hold a neighbour of any of
 // its rows, so the sweep skips it (its copies, products and epilogue).  Ties stay
 // exact: a skipped column is strictly farther than the bound.  Used for plain
@@ -3178,7 +3188,7 @@ int run_shard_knn(const void* X, int64_t N, int d, int dtype, const uint32_t* me
     const bool skip_f32 =
         dtype == ANN_F32 && pl.rerank && d <= 200 && (split_keys || bf16_keys || f16_keys);
     if (w.tlist && tile_prune_on() && (skip_u8 || skip_f32)) {
-        // 3a. bounds: each row's k'-th distance within its 256-row window (k' = the
+        // 3a. bounds: each row's k'-th distance within its 512-row window (k' = the
         // list width), the centre and radius of every 128-row group, and each block's
         // list of the tiles that may hold a neighbour, nearest first
         const int64_t ng = w.rows_cap / kt::BM;
