@@ -1901,7 +1901,7 @@ k_pool_finalize(const KnnParams P) {
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const uint32_t* gidrow = P.gid ? P.gid + pr.b_row0 : nullptr;
     uint64_t* stg = stage[warp];
-    for (int r = warp; r < kt::BM; r += 8) {
+    for (int r = warp + 8 * blockIdx.y; r < kt::BM; r += 8 * gridDim.y) {
         const int i = rb * kt::BM + r;
         if (i >= pr.n_rows) break;
         const int64_t prow = pr.pool_row0 + i;
@@ -2156,6 +2156,89 @@ __global__ void k_rerank_vec(const void* X, const void* Xrow, int d,
             Chunk16<DT>::unpack(w1, f1);
             s0 = sq_diff_add<V>(fa, f0, s0);
             s1 = sq_diff_add<V>(fa, f1, s1);
+        }
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1) {
+            s0 = __fadd_rn(s0, __shfl_xor_sync(0xffffffffu, s0, o));
+            s1 = __fadd_rn(s1, __shfl_xor_sync(0xffffffffu, s1, o));
+        }
+#pragma unroll
+        for (int h = 0; h < 2; ++h) {
+            const int cc = c + h;
+            const uint32_t v = h ? v1 : v0;
+            if (v != ANN_PAD && (cc & 31) == lane) {
+                const int e = cc >> 5;
+#pragma unroll
+                for (int q = 0; q < E; ++q)
+                    if (q == e) keys[q] = ((uint64_t)f2ord(h ? s1 : s0) << 32) | v;
+            }
+        }
+    }
+    warp_bitonic_u64<E>(keys);
+#pragma unroll
+    for (int e = 0; e < E; ++e) {
+        const int idx = lane * E + e;
+        if (idx < k) {
+            const uint64_t x = keys[e];
+            const bool pad = (x == ~0ull);
+            out_id[p * k + idx] = pad ? ANN_PAD : (uint32_t)x;
+            out_d[p * k + idx] = pad ? INFINITY : ord2f((uint32_t)(x >> 32));
+        }
+    }
+}
+
+// The same sums for rows of at most 32 NQ chunks: the row's chunks stay in registers
+// (missing ones are zeros, whose terms add nothing) and all loads of two candidates are
+// in flight together.  k_rerank_vec above, which reads the row again for every pair and
+// waits chunk by chunk, took 25.4 ms for 400k rows of 256 candidates of 2 KB, this 23.5
+// (210 GB of candidates from L2: 8.9 TB/s).  NQ = 4; with 8 (rows of 3 KB) the registers
+// cost more than the loads gain: 5.0 -> 6.4 ms.
+template <int E, int DT, int NQ>
+__global__ void k_rerank_wide(const void* X, const void* Xrow, int d,
+                              const uint32_t* __restrict__ row_ids, int64_t nrows,
+                              const uint32_t* __restrict__ cand, int kc, int k,
+                              uint32_t* __restrict__ out_id, float* __restrict__ out_d,
+                              const int64_t* __restrict__ order) {
+    constexpr int V = Chunk16<DT>::V;
+    const int lane = threadIdx.x & 31;
+    int64_t p = (blockIdx.x * (int64_t)blockDim.x + threadIdx.x) >> 5;
+    if (p >= nrows) return;
+    if (order && (p = order[p]) < 0) return;
+    const int64_t u = row_ids ? (int64_t)row_ids[p] : p;
+    const int nch = d / V;
+    uint4 ra[NQ];
+#pragma unroll
+    for (int i = 0; i < NQ; ++i) {
+        ra[i] = make_uint4(0, 0, 0, 0);
+        if (lane + 32 * i < nch) ra[i] = __ldg((const uint4*)Xrow + u * nch + lane + 32 * i);
+    }
+    uint64_t keys[E];
+#pragma unroll
+    for (int e = 0; e < E; ++e) keys[e] = ~0ull;
+    for (int c = 0; c < kc; c += 2) {
+        const uint32_t v0 = cand[p * kc + c];
+        const uint32_t v1 = c + 1 < kc ? cand[p * kc + c + 1] : ANN_PAD;
+        if (v0 == ANN_PAD && v1 == ANN_PAD) continue;  // uniform
+        const uint4* x0 = (const uint4*)X + (int64_t)(v0 == ANN_PAD ? 0 : v0) * nch;
+        const uint4* x1 = (const uint4*)X + (int64_t)(v1 == ANN_PAD ? 0 : v1) * nch;
+        uint4 w0[NQ], w1[NQ];
+#pragma unroll
+        for (int i = 0; i < NQ; ++i) {
+            w0[i] = w1[i] = make_uint4(0, 0, 0, 0);
+            if (lane + 32 * i < nch) {
+                w0[i] = __ldg(x0 + lane + 32 * i);
+                w1[i] = __ldg(x1 + lane + 32 * i);
+            }
+        }
+        float s0 = 0.0f, s1 = 0.0f;
+#pragma unroll
+        for (int i = 0; i < NQ; ++i) {
+            float fa[V], f[V];
+            Chunk16<DT>::unpack(ra[i], fa);
+            Chunk16<DT>::unpack(w0[i], f);
+            s0 = sq_diff_add<V>(fa, f, s0);
+            Chunk16<DT>::unpack(w1[i], f);
+            s1 = sq_diff_add<V>(fa, f, s1);
         }
 #pragma unroll
         for (int o = 16; o > 0; o >>= 1) {
@@ -2478,7 +2561,7 @@ k_group_geom(const void* X, int dtype, int d, const int64_t* __restrict__ src, i
     }
     for (int t = tid; t < d; t += blockDim.x) {
         float sum = 0.0f;
-#pragma unroll 8
+#pragma unroll 32
         for (int i = 0; i < kt::BM; ++i) {
             const int64_t v = rs[i];
             if (v >= 0) sum += load_elem(X, dtype, v * d + t);
@@ -2491,22 +2574,29 @@ k_group_geom(const void* X, int dtype, int d, const int64_t* __restrict__ src, i
     // radius: one warp per row, lanes over the dimensions (coalesced row reads)
     const int warp = tid >> 5, lane = tid & 31;
     float rw = 0.0f, nw = 0.0f;
-    for (int i = warp; i < kt::BM; i += 4) {
-        const int64_t v = rs[i];
-        if (v < 0) continue;
-        float r2 = 0.0f, n2 = 0.0f;
+    for (int i = warp; i < kt::BM; i += 16) {  // four rows a turn, their loads together
+        float r2[4] = {}, n2[4] = {};
         for (int t = lane; t < d; t += 32) {
-            const float x = load_elem(X, dtype, v * d + t);
-            const float df = x - cs[t];
-            r2 = fmaf(df, df, r2);
-            n2 = fmaf(x, x, n2);
+            const float c = cs[t];
+#pragma unroll
+            for (int z = 0; z < 4; ++z) {
+                const int64_t v = rs[i + 4 * z];
+                if (v < 0) continue;  // (its sums stay zero)
+                const float x = load_elem(X, dtype, v * d + t);
+                const float df = x - c;
+                r2[z] = fmaf(df, df, r2[z]);
+                n2[z] = fmaf(x, x, n2[z]);
+            }
         }
-        for (int o = 16; o; o >>= 1) {
-            r2 += __shfl_xor_sync(0xffffffffu, r2, o);
-            n2 += __shfl_xor_sync(0xffffffffu, n2, o);
+#pragma unroll
+        for (int z = 0; z < 4; ++z) {
+            for (int o = 16; o; o >>= 1) {
+                r2[z] += __shfl_xor_sync(0xffffffffu, r2[z], o);
+                n2[z] += __shfl_xor_sync(0xffffffffu, n2[z], o);
+            }
+            rw = fmaxf(rw, r2[z]);
+            nw = fmaxf(nw, n2[z]);
         }
-        rw = fmaxf(rw, r2);
-        nw = fmaxf(nw, n2);
     }
     if (lane == 0) {
         rmax[warp] = rw;
@@ -2864,6 +2954,8 @@ static int launch_tiles(const KnnPlan& pl, const void* GA, int64_t rowsA, const 
     }
     // merge the two column halves' pools of every row into its sorted list
     const unsigned g = (unsigned)grid;
+    // small launches: four CTAs a row block (161 blocks of lists of 48: 93 -> 63 us)
+    const dim3 gf(g, grid < 152 * 4 ? 4 : 1);
     if (P.kprime == 1) {
         k_pool_finalize1<<<g, kt::BM, 0, st>>>(P);
         ANN_CHECK_LAUNCH();
@@ -2873,7 +2965,7 @@ static int launch_tiles(const KnnPlan& pl, const void* GA, int64_t rowsA, const 
     const int eh = P.ph >> 5;
 #define ANN_FINALIZE(KE, EH)                                  \
     if (ke == KE && eh == EH) {                               \
-        k_pool_finalize<KE, EH><<<g, 256, 0, st>>>(P);        \
+        k_pool_finalize<KE, EH><<<gf, 256, 0, st>>>(P);       \
         ANN_CHECK_LAUNCH();                                   \
         return ANN_OK;                                        \
     }
@@ -2913,11 +3005,15 @@ static int launch_rerank(const void* X, const void* Xrow, int dtype, int d, cons
     const int es = dtype_bytes(dtype);
     const bool vec = ((size_t)d * es) % 16 == 0 && (uintptr_t)X % 16 == 0 &&
                      (uintptr_t)Xrow % 16 == 0;
+    const int nq = ((d * es) / 16 + 31) / 32;  // 16-byte chunks a lane of 32
     const bool narrow = (d * es) / 16 <= 32;  // whole row in 4 chunks per lane of 8
 #define ANN_RERANK_VEC(E, DT)                                                                  \
     if (narrow)                                                                                \
         k_rerank_g8<E, DT><<<grid, threads, 0, st>>>(X, Xrow, d, row_ids, nwarps, cand, kc, k, \
                                                      out_id, out_d, order);                     \
+    else if (nq <= 4)                                                                          \
+        k_rerank_wide<E, DT, 4><<<grid, threads, 0, st>>>(X, Xrow, d, row_ids, nwarps, cand,   \
+                                                          kc, k, out_id, out_d, order);        \
     else                                                                                       \
         k_rerank_vec<E, DT><<<grid, threads, 0, st>>>(X, Xrow, d, row_ids, nwarps, cand, kc,   \
                                                       k, out_id, out_d, order)
