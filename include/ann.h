@@ -125,8 +125,8 @@ int ann_timing_read(double* tile_ms, int* launches);
  * MMA wait-for-data cycles, MMA wait-for-accumulator cycles, producer wait
  * cycles, CTA cycles, CTAs, TMEM-load wait cycles, filter cycles, append cycles
  * (everything after the filter, compactions included), MMA issue cycles, MMA
- * commit cycles, MMA loop cycles, stash-write cycles, cycles appending chunks
- * straight to the pools, cycles moving the stash to the pools. */
+ * commit cycles, MMA loop cycles, (unused, 0), cycles storing survivors to the
+ * pools, (unused, 0). */
 int ann_tile_counters_enable(int on);
 int ann_tile_counters_read(unsigned long long* out, int n);
 

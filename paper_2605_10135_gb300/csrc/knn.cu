@@ -2515,7 +2515,7 @@ static inline size_t row_bytes(const KnnPlan& pl) { return (size_t)pl.Kp * (pl.e
 // k-th squared distance from above (the window mode of the tile kernel: one tile a row
 // block on the tensor cores and a search of its keys; direct distances with dp4a or
 // 8 x 8 FP32 register tiles took 5.2 ms for 2M uint8 rows of 128 and 84 ms for 20M FP32
-// rows of 96, this about 2 and 18 ms); a column tile whose
+// rows of 96, this 2.7 and 23.5 ms); a column tile whose
 // groups all lie beyond the block's largest bound cannot hold a neighbour of any of
 // its rows, so the sweep skips it (its copies, products and epilogue).  Ties stay
 // exact: a skipped column is strictly farther than the bound.  Used for plain
