@@ -2512,7 +2512,7 @@ static inline size_t row_bytes(const KnnPlan& pl) { return (size_t)pl.Kp * (pl.e
 // the same shard), with centres c_A, c_G and radii r_A >= max |x - c_A|, r_G, every
 // pair satisfies |x - y| >= |c_A - c_G| - r_A - r_G (triangle inequality).  The k-th
 // distance of each row among the other rows of its 512-row window bounds its final
-// k-th squared distance from above (the window mode of the tile kernel: one tile a row
+// k-th squared distance from above (the window mode of the tile kernel: two tiles a row
 // block on the tensor cores and a search of its keys; direct distances with dp4a or
 // 8 x 8 FP32 register tiles took 5.2 ms for 2M uint8 rows of 128 and 84 ms for 20M FP32
 // rows of 96, this 2.7 and 23.5 ms); a column tile whose
