@@ -306,7 +306,11 @@ __device__ __forceinline__ bool bound_keeps(const Bound& T, uint64_t v, const ui
 // value): two around the place where the wanted rank falls if the keys between lo and
 // hi are spread evenly, one in the middle of what lies above.  It stops as soon as the
 // keys at or below a pivot number kp to maxkeep: two or three steps for spread keys,
-// where halving the range of the key bits takes nine or more.  Only when more than
+// where halving the range of the key bits takes nine or more.  Where that place cannot be
+// computed (hi - lo beyond FP32's range, an infinite key) or eight steps were not enough
+// (ties, keys of very different size), the pivots quarter and halve the bits that are
+// left, at most 32 more steps: interpolation alone took 223 steps for 256 keys of three
+// values around zero, and with hi - lo = inf it came down by one bit a step.  Only when more than
 // maxkeep entries share the kp-th key are their global ids searched (then exactly kp
 // stay).
 template <int E>
@@ -325,13 +329,17 @@ __device__ __forceinline__ Bound warp_select(const uint64_t (&v)[E], int n, int 
     // invariant: #{key <= hi} = chi >= kp, #{key < lo} = clo < kp
     uint32_t lo = kmin, hi = kmax;
     int chi = n, clo = 0;
+    int interp = 8;
     while (chi > maxkeep && lo < hi) {
         // pivots lie in [lo, hi); interpolated on the key values (on their bits a range
-        // across zero is exponential), the last one halves the bits that are left, so
-        // every step makes progress
+        // across zero is exponential), the last one halves the bits that are left
         const float f = (0.5f * (float)(kp + maxkeep) - (float)clo) / (float)(chi - clo);
         const float flo = ord2f(lo), fw = ord2f(hi) - flo;
         uint32_t p1 = f2ord(fmaf(0.8f * f, fw, flo)), p2 = f2ord(fmaf(1.2f * f, fw, flo));
+        if (__builtin_expect(--interp < 0 || !(fw < INFINITY), 0)) {
+            p1 = lo + ((hi - lo) >> 2);
+            p2 = lo + ((hi - lo) >> 1);
+        }
         p1 = p1 < lo ? lo : p1 > hi - 1 ? hi - 1 : p1;
         p2 = p2 < p1 ? p1 : p2 > hi - 1 ? hi - 1 : p2;
         const uint32_t p3 = hi - 1 - ((hi - 1 - p2) >> 1);
