@@ -187,7 +187,7 @@ struct KnnParams {
 // frees 120 of them, of 320 only 56); always at least 32 more than k' (a chunk's
 // survivors fit after a compaction).  A larger pool compacts less often at about the
 // same cost per compaction.
-__host__ __device__ inline int pool_half(int kprime, bool rerank) {
+__host__ __device__ constexpr int pool_half(int kprime, bool rerank) {
     int ph = kprime < 32 ? 2 * kprime : kprime <= 128 ? 256 : kprime + 64;
     if (ph < kprime + 32) ph = kprime + 32;
     ph = (ph + 31) / 32 * 32;
@@ -2911,6 +2911,32 @@ size_t knn_ws(int C, int64_t rows, const KnnPlan& pl, KnnWs* out, void* base, si
     return cv.used + 256;
 }
 
+// The instantiations of k_pool_finalize: sorted entries a lane for the list width, pool
+// entries a lane and half.  Every list width of 2 to 256, re-ranked or not, has its own,
+// and each is some width's.
+#define ANN_FINALIZE_SIZES(X)                                                                 \
+    X(1, 2) X(1, 8) X(2, 8) X(4, 8) X(8, 7) X(8, 8) X(8, 9) X(8, 10) X(8, 11) X(8, 12)
+constexpr int finalize_ke(int kprime) {
+    return kprime <= 32 ? 1 : kprime <= 64 ? 2 : kprime <= 128 ? 4 : 8;
+}
+constexpr bool finalize_sizes_match() {
+    bool used[9][13] = {};
+    for (int kp = 2; kp <= 256; ++kp)
+        for (int rerank = 0; rerank < 2; ++rerank)
+            used[finalize_ke(kp)][pool_half(kp, rerank != 0) / 32] = true;
+#define ANN_FINALIZE(KE, EH)           \
+    if (!used[KE][EH]) return false;   \
+    used[KE][EH] = false;
+    ANN_FINALIZE_SIZES(ANN_FINALIZE)
+#undef ANN_FINALIZE
+    for (auto& row : used)
+        for (bool u : row)
+            if (u) return false;
+    return true;
+}
+static_assert(finalize_sizes_match(), "k_pool_finalize: a list width without an instantiation, "
+                                      "or an instantiation without a list width");
+
 static int launch_tiles(const KnnPlan& pl, const void* GA, int64_t rowsA, const void* ones,
                         const void* GB, const void* augB, int64_t rowsB, const KnnParams& P,
                         int64_t grid, cudaStream_t st, bool timed) {
@@ -2969,31 +2995,14 @@ static int launch_tiles(const KnnPlan& pl, const void* GA, int64_t rowsA, const 
         ANN_CHECK_LAUNCH();
         return ANN_OK;
     }
-    const int ke = P.kprime <= 32 ? 1 : P.kprime <= 64 ? 2 : P.kprime <= 128 ? 4 : 8;
-    const int eh = P.ph >> 5;
+    const int ke = finalize_ke(P.kprime), eh = P.ph >> 5;
 #define ANN_FINALIZE(KE, EH)                                  \
     if (ke == KE && eh == EH) {                               \
         k_pool_finalize<KE, EH><<<gf, 256, 0, st>>>(P);       \
         ANN_CHECK_LAUNCH();                                   \
         return ANN_OK;                                        \
     }
-    ANN_FINALIZE(1, 2)
-    ANN_FINALIZE(1, 8)
-
-    ANN_FINALIZE(2, 3)
-    ANN_FINALIZE(2, 4)
-    ANN_FINALIZE(2, 6)
-    ANN_FINALIZE(2, 8)
-
-    ANN_FINALIZE(4, 5)
-    ANN_FINALIZE(4, 6)
-    ANN_FINALIZE(4, 7)
-    ANN_FINALIZE(4, 8)
-    ANN_FINALIZE(8, 7)
-    ANN_FINALIZE(8, 8)
-    ANN_FINALIZE(8, 9)
-    ANN_FINALIZE(8, 10)
-    ANN_FINALIZE(8, 12)
+    ANN_FINALIZE_SIZES(ANN_FINALIZE)
 #undef ANN_FINALIZE
     return fail(ANN_ERR_UNSUPPORTED, "tile launch: no finalize for k' = %d, pool %d", P.kprime,
                 P.ph);
