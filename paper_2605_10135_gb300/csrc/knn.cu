@@ -3355,12 +3355,12 @@ int run_shard_knn(const void* X, int64_t N, int d, int dtype, const uint32_t* me
 // without thresholds, which costs it about six tiles.  1,000 queries over 1M uint8
 // vectors (8 row blocks): 8 CTAs of 3,907 tiles took 5.6 ms, 152 of 206 take 0.74 ms
 // (a range meets more survivors than the whole: k' (1 + ln(n / k')) a range).
-constexpr int QS_MAX = 32;
+constexpr int QS_MAX = 32, QS_BLOCKS = 2 * 152;  // ranges; row blocks x ranges, if split
 static int query_splits(int64_t N, int64_t nq) {
     const int64_t nb = (nq + kt::BM - 1) / kt::BM, tiles = (N + kt::BNMAX - 1) / kt::BNMAX;
     int best = 1;
     double cost = 0.0;
-    for (int ns = 1; ns <= QS_MAX && ns <= tiles && (ns == 1 || nb * ns <= 2 * 152); ++ns) {
+    for (int ns = 1; ns <= QS_MAX && ns <= tiles && (ns == 1 || nb * ns <= QS_BLOCKS); ++ns) {
         const int64_t per = (tiles + ns - 1) / ns;
         const double c = (double)((nb * ns + 151) / 152) * (double)(per + 6);
         if (ns == 1 || c < cost) {
@@ -3369,6 +3369,16 @@ static int query_splits(int64_t N, int64_t nq) {
         }
     }
     return best;
+}
+// Pool rows that hold the splits of nq queries and of any smaller number (0: a single
+// column tile, never split): the scratch reported for nq grows with nq, so scratch sized for
+// one launch also serves a smaller one, which may be split further (1,000 queries over 20k
+// vectors take 16 ranges, 15,000 take one).
+static int64_t split_rows(int64_t N, int64_t nq) {
+    const int64_t tiles = (N + kt::BNMAX - 1) / kt::BNMAX;
+    const int64_t most = tiles < QS_MAX ? tiles : QS_MAX;
+    const int64_t rows = most * ((nq + kt::BM - 1) / kt::BM * kt::BM);
+    return most < 2 ? 0 : rows < QS_BLOCKS * kt::BM ? rows : QS_BLOCKS * kt::BM;
 }
 size_t query_ws(int64_t N, int64_t nq, const KnnPlan& pl, QueryWs* out, void* base, size_t cap) {
     Carver cv(base, cap);
@@ -3390,10 +3400,11 @@ size_t query_ws(int64_t N, int64_t nq, const KnnPlan& pl, QueryWs* out, void* ba
     w.cand_id = pl.rerank ? cv.take<uint32_t>((size_t)nq * pl.kprime) : nullptr;
     w.ns = ns;
     w.pstride = ns > 1 ? (nq + kt::BM - 1) / kt::BM * kt::BM : 0;
-    const int64_t prows = ns > 1 ? ns * w.pstride : w.capA;
+    const int64_t srows = split_rows(N, nq), prows = w.capA > srows ? w.capA : srows;
     w.pool = cv.take<uint64_t>((size_t)prows * 2 * pool_half(pl.kprime, pl.rerank));
     w.pool_cnt = cv.take<int>((size_t)prows * 2);
-    w.split_list = ns > 1 ? cv.take<uint64_t>((size_t)prows * pl.kprime) : nullptr;
+    w.split_list = srows ? cv.take<uint64_t>((size_t)srows * pl.kprime) : nullptr;
+    if (ns == 1) w.split_list = nullptr;
     w.srcA = cv.take<int64_t>((size_t)w.capA);
     w.srcB = cv.take<int64_t>((size_t)w.capB);
     w.amax = cv.take<float>(4);

@@ -162,8 +162,8 @@ struct QueryWs {
     int ns;             // column splits
     int64_t pstride;    // pool rows of one split (ns > 1)
     uint64_t* pool;     // [rows x 2 x pool_half] candidate pools of the sweep
-    int* pool_cnt;      // [rows x 2], rows = ns pstride (capA without splits)
-    uint64_t* split_list;  // [rows x kprime] sorted lists of the splits (ns > 1)
+    int* pool_cnt;      // [rows x 2], ns pstride rows used (nq without splits)
+    uint64_t* split_list;  // [rows x kprime] sorted lists of the splits (NULL: ns = 1)
     int64_t capA, capB;
     int64_t* srcA;
     int64_t* srcB;
