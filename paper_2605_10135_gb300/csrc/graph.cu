@@ -5,10 +5,10 @@
 // Prune, one warp per shard row u: u's list goes into an id -> position table
 // in shared memory (one probe per lookup, a multiplier chosen per row so that
 // no two of its ids share a slot); the lists of u's neighbours are read with
-// coalesced warp loads, every entry looked up, and the counts c_j kept in
-// shared memory (one predicated add per entry).  The R entries of smallest
-// (c_j, j) are chosen by a warp bitonic sort and written in list order with a
-// ballot/popc compaction.  Integer logic only.
+// coalesced warp loads, every entry looked up, and the counts c_j kept as bits,
+// one per neighbour, in shared memory (one predicated OR per entry).  The R
+// entries of smallest (c_j, j) are chosen by a warp bitonic sort and written in
+// list order with a ballot/popc compaction.  Integer logic only.
 //
 // Merge, one warp per vector g: its pruned lists (one per shard holding g) are
 // gathered, sorted by (id, distance) to drop duplicate ids (the smaller
@@ -106,24 +106,25 @@ __device__ __forceinline__ uint32_t tmult(int a) { return HM + 0x3C6EF372u * (ui
 __device__ __forceinline__ uint32_t tkey(uint32_t y) { return y << 10; }  // low 22 bits << 10
 
 // Shared memory of one prune warp: table words [TS], the neighbours' rows [KM], overflow
-// ids and positions [KM each], the counts [KM], the overflow count (+pad).
+// ids and positions [KM each], the hit bits [KM / 32][KM], the overflow count (+pad).
 __host__ __device__ constexpr size_t prune_warp_smem(int KM) {
-    return (size_t)TS * 4 + (size_t)KM * 20 + 16;
+    return (size_t)TS * 4 + (size_t)KM * 16 + (size_t)(KM / 32) * KM * 4 + 16;
 }
 
 // Detour counts of one row: for each neighbour v_i (i < m) the warp reads L_{v_i}
 // with coalesced loads (entry t in lane t % 32, register t / 32) and looks each
 // entry up in u's table; an entry at position j of u's list with i < j and t < j
-// adds one to cnt[j] (the ids of a list are distinct: one add per (i, j) pair).  Bound
-// by instruction issue: a lookup is a multiply, a table read, two compares and the
-// add.  Collecting the hits as bits of 64-bit words and OR-reducing them over the
-// warp for each neighbour took more instructions, and a compare-and-swap per id and
-// try of the table cost as much again (12.8 ms for 2M rows of 64, this 11.4).
+// sets bit i of hit[.][j], so that a neighbour whose list holds an id twice counts once;
+// c_j is the number of bits.  Bound by instruction issue: a lookup is a multiply, a table
+// read, two compares and the shared-memory OR.  Collecting the hits as bits of 64-bit
+// words and OR-reducing them over the warp for each neighbour took more instructions,
+// and a compare-and-swap per id and try of the table cost as much again (12.8 ms for 2M
+// rows of 64, this 11.4).
 template <int E, bool OVF>
 __device__ __forceinline__ void prune_counts(const uint32_t* __restrict__ knn_id, int k, int m,
                                              const int64_t* wrow, const uint32_t* tw,
                                              const uint32_t* ovf, const uint32_t* ovf_pos,
-                                             int novf, uint32_t A, uint32_t* cnt) {
+                                             int novf, uint32_t A, uint32_t* hit) {
     constexpr int G = E <= 2 ? 8 : 2;  // neighbour lists read together (loads in flight)
     const int lane = threadIdx.x & 31;
     for (int i0 = 0; i0 + 1 < m; i0 += G) {  // (the last neighbour has no j behind it)
@@ -152,7 +153,8 @@ __device__ __forceinline__ void prune_counts(const uint32_t* __restrict__ knn_id
                     for (int o = 0; o < novf; ++o)
                         if (ovf[o] == x[g][e]) dj = ovf_pos[o];
                 }
-                if (dj - first < 256u - first) atomicAdd(cnt + dj, 1u);
+                if (dj - first < 256u - first)
+                    atomicOr(hit + (i >> 5) * (32 * E) + dj, 1u << (i & 31));
             }
         }
     }
@@ -176,8 +178,8 @@ __global__ void k_prune(const uint32_t* __restrict__ knn_id, const float* __rest
     int64_t* wrow = (int64_t*)(tw + TS);           // [KM]
     uint32_t* ovf = (uint32_t*)(wrow + KM);        // [KM]
     uint32_t* ovf_pos = ovf + KM;                  // [KM]
-    uint32_t* cnt = ovf_pos + KM;                  // [KM]
-    int* novf_p = (int*)(cnt + KM);                // [1] (+pad)
+    uint32_t* hit = ovf_pos + KM;                  // [E][KM]
+    int* novf_p = (int*)(hit + E * KM);            // [1] (+pad)
     const uint32_t lt = (1u << lane) - 1;
     // the table starts empty once; after each row only the slots its ids used are
     // emptied again
@@ -267,15 +269,19 @@ __global__ void k_prune(const uint32_t* __restrict__ knn_id, const float* __rest
             }
             uint32_t c[E];
 #pragma unroll
-            for (int e = 0; e < E; ++e) cnt[lane + 32 * e] = 0;
+            for (int w = 0; w < E * E; ++w) hit[lane + 32 * w] = 0;
             __syncwarp();
             if (novf == 0)
-                prune_counts<E, false>(knn_id, k, m, wrow, tw, ovf, ovf_pos, 0, A, cnt);
+                prune_counts<E, false>(knn_id, k, m, wrow, tw, ovf, ovf_pos, 0, A, hit);
             else
-                prune_counts<E, true>(knn_id, k, m, wrow, tw, ovf, ovf_pos, novf, A, cnt);
+                prune_counts<E, true>(knn_id, k, m, wrow, tw, ovf, ovf_pos, novf, A, hit);
             __syncwarp();
 #pragma unroll
-            for (int e = 0; e < E; ++e) c[e] = cnt[lane + 32 * e];
+            for (int e = 0; e < E; ++e) {
+                c[e] = 0;
+#pragma unroll
+                for (int w = 0; w < E; ++w) c[e] += __popc(hit[w * KM + lane + 32 * e]);
+            }
             // rank positions by (c_j, j); any starting placement sorts the same
             uint32_t sel[E];
 #pragma unroll
