@@ -455,7 +455,10 @@ __device__ __forceinline__ void epi_compact(EpiState& s, uint32_t mask) {
             T = warp_select(v, cr, want, most, s.gidrow);
             if (want == s.kp) break;
             const float own = fminf(ord2f(T.key), s.q_own[r]);
-            const uint32_t t = f2ord(fmaxf(own, s.q_other[r]));
+            // the other half's warp may be lowering its bound: one lane's copy for all, so
+            // that the entries kept and the threshold set below follow the same bound
+            const float other = __shfl_sync(0xffffffffu, s.q_other[r], 0);
+            const uint32_t t = f2ord(fmaxf(own, other));
             int n = 0;
 #pragma unroll
             for (int e = 0; e < EM; ++e) n += (uint32_t)(v[e] >> 32) <= t && v[e] != ~0ull;
