@@ -124,22 +124,22 @@ int ann_timing_read(double* tile_ms, int* launches);
  * with survivors, compactions, rows compacted, (unused, 0), appended survivors,
  * MMA wait-for-data cycles, MMA wait-for-accumulator cycles, producer wait
  * cycles, CTA cycles, CTAs, TMEM-load wait cycles, filter cycles, append cycles
- * (everything after the filter, compactions included), MMA issue cycles, MMA
- * commit cycles, MMA loop cycles, (unused, 0), cycles storing survivors to the
+ * (everything after the filter, compactions included), MMA issue cycles (a
+ * stage's commit included), (unused, 0), MMA loop cycles, (unused, 0), cycles storing survivors to the
  * pools, (unused, 0). */
 int ann_tile_counters_enable(int on);
 int ann_tile_counters_read(unsigned long long* out, int n);
 
 /* Exact skipping of distance tiles (on by default).  For ANN_EXACT on uint8
- * vectors of d <= 256 (d a multiple of 4, X 4-byte aligned) and on float32 vectors
- * of d <= 200, each
- * row's k'-th squared distance among the rows of its 512-row window of the shard
- * (k' = the screened list width) bounds its final one from above; where the tile
- * keys are not exact the bound also carries a margin for their error.  A column tile is then
+ * vectors of d <= 256 (d a multiple of 4, X 4-byte aligned) and for float32 vectors
+ * of d <= 200 (exact, BF16 and FP16 forms), each row's k'-th tile key among the rows of
+ * its window of the shard (the two column tiles that hold its block, 512 or 256 rows;
+ * k' = the screened list width) bounds its final one from above.  A column tile is then
  * skipped (no copy, no product, no epilogue) when the triangle inequality over
  * 128-row groups (centre and radius bound of each group) shows that every column
- * in it is strictly farther than the block's largest bound.  The lists do not
- * change (ties included).  ann_tile_prune(0) sweeps every tile.
+ * in it is strictly farther than the block's largest bound (where the tile keys are
+ * not exact, by more than their error).  The lists do not change (ties included).
+ * ann_tile_prune(0) sweeps every tile.
  * ann_tile_prune_stats synchronises the device, writes up to n counters to host
  * out[] and clears them: column tiles of the blocks, tiles swept, (row, column)
  * pairs swept. */

@@ -182,13 +182,13 @@ def tile_counters_read() -> dict:
 
 
 def tile_prune(on: bool = True):
-    """Switch the exact pruning of distance tiles (uint8, ANN_EXACT) on or off."""
+    """Switch the exact skipping of distance tiles (uint8 and float32; see ann.h) on or off."""
     _check(lib().ann_tile_prune(1 if on else 0))
 
 
 def tile_prune_stats() -> dict:
-    """Counts since the last read (synchronises the device): half-tiles of the
-    launches, half-tiles examined, (row, column) pairs examined."""
+    """Counts since the last read (synchronises the device): column tiles of the
+    blocks, tiles swept, (row, column) pairs swept."""
     arr = (ct.c_ulonglong * 3)()
     _check(lib().ann_tile_prune_stats(arr, 3))
     return dict(tiles=int(arr[0]), swept=int(arr[1]), pairs=int(arr[2]))

@@ -119,7 +119,7 @@ __host__ __device__ constexpr size_t prune_warp_smem(int KM) {
 // read, two compares and the shared-memory OR.  Collecting the hits as bits of 64-bit
 // words and OR-reducing them over the warp for each neighbour took more instructions,
 // and a compare-and-swap per id and try of the table cost as much again (12.8 ms for 2M
-// rows of 64, this 11.4).
+// rows of 64, this 11.7).
 template <int E, bool OVF>
 __device__ __forceinline__ void prune_counts(const uint32_t* __restrict__ knn_id, int k, int m,
                                              const int64_t* wrow, const uint32_t* tw,

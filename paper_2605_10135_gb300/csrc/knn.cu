@@ -18,11 +18,14 @@
 //              ring of stages (one 128-byte K block, 128-byte swizzle) and their
 //              16-element norm blocks through a second, small ring (32-byte
 //              swizzle).
-//   warp 1   : allocates 512 TMEM columns (two FP32 accumulators) and issues
-//              tcgen05.mma (M=128, N=256 or 128, K=16; K=32 for E4M3) from one
-//              thread.  The issue of an MMA waits for room in the tensor pipe, so
-//              the thread does little else: one commit per stage and one per tile.
-//   warps 2-9: epilogue, two warps per TMEM lane quarter (one thread per row,
+//   warp 1   : allocates 512 TMEM columns (two FP32 accumulators); the whole warp
+//              walks the tiles and takes the waits, one elected lane issues
+//              tcgen05.mma (M=128, N=256 or 128, K=16; K=32 for E4M3).  The issue of
+//              an MMA waits for room in the tensor pipe, so the lane does little
+//              else: one commit per stage and one per tile.
+//   warps 2-3: idle; they fill up the warpgroup that gives its registers to the
+//              epilogue (setmaxnreg).
+//   warps 4-11: epilogue, two warps per TMEM lane quarter (one thread per row,
 //              one column half per warp).  32-column chunks are read with
 //              tcgen05.ld (the next chunk's load overlaps the current chunk's
 //              work) and reduced with 3-input minima; a chunk is skipped unless
@@ -92,17 +95,17 @@ enum TileCounter {
     TC_FLUSH_ITERS,      // warp-level: rows compacted
     TC_INSERTS,          // thread-level: pool entries left after compactions (unused: 0)
     TC_APPENDS,          // thread-level: survivors appended to the pools
-    TC_MMA_WAIT_FULL,    // MMA thread: cycles waiting for B stages
-    TC_MMA_WAIT_ACC,     // MMA thread: cycles waiting for a free accumulator
+    TC_MMA_WAIT_FULL,    // MMA warp: cycles waiting for B stages
+    TC_MMA_WAIT_ACC,     // MMA warp: cycles waiting for a free accumulator
     TC_PROD_WAIT,        // producer: cycles waiting for a free stage
     TC_CTA_CYCLES,       // thread 0: cycles from start to teardown
     TC_CTAS,             // CTAs that ran
     TC_LD_WAIT,          // epilogue threads: cycles blocked in tcgen05.wait::ld
     TC_FILTER,           // epilogue threads: cycles in the chunk filter (min + vote)
     TC_APPEND,           // epilogue threads: cycles appending survivors (incl. flush)
-    TC_MMA_ISSUE,        // MMA thread: cycles issuing tcgen05.mma
-    TC_MMA_COMMIT,       // MMA thread: cycles in tcgen05.commit
-    TC_MMA_LOOP,         // MMA thread: cycles from the A wait to the end of the tile loop
+    TC_MMA_ISSUE,        // MMA warp: cycles issuing tcgen05.mma and a stage's commit
+    TC_MMA_COMMIT,       // (unused: 0)
+    TC_MMA_LOOP,         // MMA warp: cycles from the A wait to the end of the tile loop
     TC_STASH,            // (unused: 0)
     TC_DIRECT,           // epilogue threads: cycles storing a chunk's survivors to the pools
     TC_FLUSH_LOOP,       // (unused: 0)
@@ -300,9 +303,9 @@ __device__ __forceinline__ bool bound_keeps(const Bound& T, uint64_t v, const ui
     return column_gid(gidrow, (uint32_t)v) <= T.id;
 }
 
-// A bound that keeps between kp and maxkeep of a warp's n <= 640 entries (E per lane;
-// n > maxkeep >= kp), exactly kp when maxkeep == kp.  Each step counts the keys at or
-// below three pivots (10 bits each of one warp sum, so all lanes return the same
+// A bound that keeps between kp and maxkeep of a warp's n <= 2 PH_MAX entries (E per
+// lane; n > maxkeep >= kp), exactly kp when maxkeep == kp.  Each step counts the keys at
+// or below three pivots (10 bits each of one warp sum, so all lanes return the same
 // value): two around the place where the wanted rank falls if the keys between lo and
 // hi are spread evenly, one in the middle of what lies above.  It stops as soon as the
 // keys at or below a pivot number kp to maxkeep: two or three steps for spread keys,
@@ -310,9 +313,10 @@ __device__ __forceinline__ bool bound_keeps(const Bound& T, uint64_t v, const ui
 // computed (hi - lo beyond FP32's range, an infinite key) or eight steps were not enough
 // (ties, keys of very different size), the pivots quarter and halve the bits that are
 // left, at most 32 more steps: interpolation alone took 223 steps for 256 keys of three
-// values around zero, and with hi - lo = inf it came down by one bit a step.  Only when more than
-// maxkeep entries share the kp-th key are their global ids searched (then exactly kp
-// stay).
+// values around zero, and with hi - lo = inf it came down by one bit a step.  Only when
+// more than maxkeep entries share the kp-th key are their global ids searched (then
+// exactly kp stay).
+static_assert(2 * kt::PH_MAX < 1024, "warp_select packs its counts in 10 bits each");
 template <int E>
 __device__ __forceinline__ Bound warp_select(const uint64_t (&v)[E], int n, int kp, int maxkeep,
                                              const uint32_t* gidrow) {
@@ -489,7 +493,8 @@ __device__ __forceinline__ void epi_compact(EpiState& s, uint32_t mask) {
 }
 
 // The kp-th smallest of a thread's 32 keys (kp <= 32; NaN = +inf), by a sorting network
-// in registers (240 exchanges, one row per lane).
+// (240 exchanges, one row per lane).  The compiler makes the pick of the kp-th an indexed
+// read, for which the sorted keys go through a 128-byte local frame.
 template <int K, int J>
 __device__ __forceinline__ void sort32_from(float (&t)[32]) {  // stages (K, J) to (32, 1)
 #pragma unroll
@@ -932,15 +937,16 @@ __global__ void __launch_bounds__(kt::THREADS, 1)
         // elected lane issues: tcgen05.mma takes its descriptors from uniform
         // registers, and under a plain "lane == 0" branch they are not known to be
         // uniform, which cost about 258 cycles an MMA whatever its width (128 x 256 x 16
-        // takes 128): 1,121 ns a tile of 9 MMAs without any epilogue, 969 now that the
-        // wait is for the operands (12 KB an MMA read and 8 KB written through the
-        // shared memory's 128 bytes a clock).
+        // takes 128): 1,121 ns a tile of 9 MMAs without any epilogue, 969 now, most of
+        // the difference to 9 x 128 clocks spent waiting for operands (72 KB from L2 a
+        // tile; neither L2 nor the shared memory is above 60% of its peak, nor is the
+        // tensor pipe).
         bool ok = mbar_wait_warp(a_bar, 0, abort_flag);
         tc_fence_after();
         int st = 0, sa = 0;
         uint32_t ph = 0, aph = 0;
         const int H2 = P.nkb_b >> 1;
-        unsigned long long w_full = 0, w_acc = 0, c_iss = 0, c_com = 0;
+        unsigned long long w_full = 0, w_acc = 0, c_iss = 0;
         long long loop0 = 0;
         if (PROF) loop0 = clock64();
         for (int t = 0; t < nrun && ok; ++t) {
@@ -1055,7 +1061,6 @@ __global__ void __launch_bounds__(kt::THREADS, 1)
             if (PROF) {
                 prof_add(TC_MMA_LOOP, (unsigned long long)(clock64() - loop0));
                 prof_add(TC_MMA_ISSUE, c_iss);
-                prof_add(TC_MMA_COMMIT, c_com);
                 prof_add(TC_MMA_WAIT_FULL, w_full);
                 prof_add(TC_MMA_WAIT_ACC, w_acc);
             }
@@ -1085,9 +1090,10 @@ __global__ void __launch_bounds__(kt::THREADS, 1)
                                               (volatile float*)(base + L.kscr));
             float ub = INFINITY;
             if (i < pr.n_rows && kb < INFINITY) {
-                // |x - y|^2 = |x|^2 + 2 key, rounded up, and the error of inexact keys (an
-                // eighth of ub_margin times |x|^2 + |y|^2 <= 3 |x|^2 + 2 dist); the scale of
-                // scaled operands is a power of two
+                // |x|^2 + 2 key, rounded up.  It bounds the sweep's keys, which are these
+                // keys bit for bit, so their distance from the true |x - y|^2 costs no
+                // neighbour; an eighth of ub_margin covers the roundings of this line.
+                // The scale of scaled operands is a power of two
                 const float nx = P.na[pr.a_row0 + i];
                 ub = fmaxf(__fmaf_ru(2.0f, kb, nx), 0.0f);
                 ub = __fmaf_ru(0.125f * P.ub_margin, __fmaf_ru(3.0f, nx, 2.0f * ub), ub);
@@ -2522,17 +2528,18 @@ static inline size_t row_bytes(const KnnPlan& pl) { return (size_t)pl.Kp * (pl.e
 // For a row block A (128 gathered rows) and a column group G (128 gathered rows of
 // the same shard), with centres c_A, c_G and radii r_A >= max |x - c_A|, r_G, every
 // pair satisfies |x - y| >= |c_A - c_G| - r_A - r_G (triangle inequality).  The k-th
-// distance of each row among the other rows of its 512-row window bounds its final
-// k-th squared distance from above (the window mode of the tile kernel: two tiles a row
+// tile key of each row among the other rows of its window, the two column tiles that
+// hold its block (512 rows with 256-wide tiles, 256 with 128-wide ones), bounds its final
+// k-th key from above (the window mode of the tile kernel: two tiles a row
 // block on the tensor cores and a search of its keys; direct distances with dp4a or
 // 8 x 8 FP32 register tiles took 5.2 ms for 2M uint8 rows of 128 and 84 ms for 20M FP32
 // rows of 96, this 2.7 and 23.5 ms); a column tile whose
 // groups all lie beyond the block's largest bound cannot hold a neighbour of any of
 // its rows, so the sweep skips it (its copies, products and epilogue).  Ties stay
-// exact: a skipped column is strictly farther than the bound.  Used for plain
-// (single-product) operands of integer data, whose tile keys are exact; every
-// rounding in the bound is pushed outward by a relative margin far above FP32's
-// error on these sums.
+// exact: a skipped column is strictly farther than the bound.  Used for uint8 data,
+// whose tile keys are exact, and for FP32 data with the margin of key_slack for the
+// keys' error; every rounding in the bound is pushed outward by a relative margin far
+// above FP32's error on these sums.
 static bool g_tile_prune = true;
 void tile_prune_set(bool on) { g_tile_prune = on; }
 bool tile_prune_on() { return g_tile_prune; }
@@ -2761,8 +2768,8 @@ k_tile_list(const int64_t* __restrict__ blk_off, const KnnProblem* __restrict__ 
                     if (ub < INFINITY) {
                         const float D =
                             sqrtf(d2 * (1.0f - (float)(d + 4) * 0x1p-22f)) * (1.0f - 0x1p-20f);
-                        // kslack (float data): twice the largest error of a tile key's
-                        // squared distance, which scales with |x|^2 + |y|^2
+                        // kslack (float data): more than the largest error of a tile
+                        // key's squared distance, which scales with |x|^2 + |y|^2
                         const float lbg = (D - rA - rg) * (1.0f - 0x1p-20f);
                         const float need =
                             ub * (1.0f + 0x1p-18f) + kslack * (gmaxn[gA] + gmaxn[g0s + c0 + g]);
@@ -3153,17 +3160,17 @@ int launch_absmax(const void* X, int dtype, int64_t n, const void* Q, int64_t nq
     return ANN_OK;
 }
 
-// Relative error of a squared distance from the tile keys, times eight (0: no bound that
-// is of use).  Split BF16 keys (three products, FP32 accumulation): the error stays below
-// (2^-16 + (d + 4) 2^-24)(|x|^2 + |y|^2), and the keys of 16-bit data, whose products are
-// exact, below the same; BF16 operands (each rounded once, relative 2^-9; the norms in
-// FP32): below (2^-8 + (d + 8) 2^-24)(|x|^2 + |y|^2); FP16 operands after an exact
-// power-of-two scale (relative 2^-11 each): below (2^-10 + (d + 8) 2^-24)(|x|^2 + |y|^2).
-static float key_slack(const KnnPlan& pl, int dtype, int d) {
+// Margin for the error of the tile keys of FP32 data, relative to |x|^2 + |y|^2 (0: no
+// bound that is of use).  A value rounded to BF16 is off by up to 2^-8 of itself, to FP16
+// (after an exact power-of-two scale) by 2^-11, and the two parts of a split value by 2^-16;
+// 2 |x| |y| <= |x|^2 + |y|^2.  So a squared distance from split keys (three products; the
+// fourth and the two remainders are left out) is off by up to 3 2^-16, from BF16 operands
+// by 2^-7, from FP16 operands by 2^-10, each plus some (d + 8) 2^-24 of FP32 accumulation.
+// A column's key has to clear the bound, itself made of keys, so one such error is enough;
+// the margin is 2.6, 4 and 8 times that.
+static float key_slack(const KnnPlan& pl, int d) {
     if (pl.elem8) return 0.0f;
-    const bool exact16 = pl.mode == 0 && !pl.scaled &&
-                         dtype == (pl.ab_fmt == 0 ? ANN_F16 : ANN_BF16);
-    if (pl.mode == 1 || exact16) return 8.0f * (0x1p-16f + (float)(d + 4) * 0x1p-24f);
+    if (pl.mode == 1) return 8.0f * (0x1p-16f + (float)(d + 4) * 0x1p-24f);
     return pl.ab_fmt == 1 ? 8.0f * (0x1p-8f + (float)(d + 8) * 0x1p-24f)
                           : 8.0f * (0x1p-10f + (float)(d + 8) * 0x1p-24f);
 }
@@ -3304,16 +3311,15 @@ int run_shard_knn(const void* X, int64_t N, int d, int dtype, const uint32_t* me
     const bool skip_f32 =
         dtype == ANN_F32 && pl.rerank && d <= 200 && (split_keys || bf16_keys || f16_keys);
     if (w.tlist && tile_prune_on() && (skip_u8 || skip_f32)) {
-        // 3a. bounds: each row's k'-th distance within its 512-row window (k' = the
-        // list width), the centre and radius of every 128-row group, and each block's
+        // 3a. bounds: each row's k'-th tile key within its window of two column tiles (k' =
+        // the list width), the centre and radius of every 128-row group, and each block's
         // list of the tiles that may hold a neighbour, nearest first
         const int64_t ng = w.rows_cap / kt::BM;
         k_group_geom<<<(unsigned)ng, 128, (size_t)d * sizeof(float), st>>>(
             X, dtype, d, w.src, ng, pl.Kp, w.gcent, w.grad, w.gmaxn);
         ANN_CHECK_LAUNCH();
         float kslack = 0.0f;
-        // a skipped column must clear the bound by twice the keys' error, taken 4x larger
-        if (!skip_u8) kslack = key_slack(pl, dtype, d);
+        if (!skip_u8) kslack = key_slack(pl, d);
         KnnParams W = P;
         W.win_rowub = w.rowub;
         W.win_bub = w.bub;
@@ -3356,7 +3362,7 @@ int run_shard_knn(const void* X, int64_t N, int d, int dtype, const uint32_t* me
 // own with pools of its own, and k_split_merge merges their sorted lists.  ns (at most
 // 32, one lane each in the merge) minimises waves x (tiles a range + 6): a range starts
 // without thresholds, which costs it about six tiles.  1,000 queries over 1M uint8
-// vectors (8 row blocks): 8 CTAs of 3,907 tiles took 5.6 ms, 152 of 206 take 0.74 ms
+// vectors (8 row blocks): 8 CTAs of 3,907 tiles took 5.6 ms, 152 of 206 take 0.79 ms
 // (a range meets more survivors than the whole: k' (1 + ln(n / k')) a range).
 constexpr int QS_MAX = 32, QS_BLOCKS = 2 * 152;  // ranges; row blocks x ranges, if split
 static int query_splits(int64_t N, int64_t nq) {

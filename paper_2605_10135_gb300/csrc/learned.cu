@@ -432,7 +432,7 @@ __device__ __forceinline__ void bf16_split(float v, __nv_bfloat16& hi, __nv_bflo
 }
 // One 32 x 32 tile per block turn, transposed through shared memory so that both forms
 // are written in runs of 64 bytes (element-wise transposed stores took 44 us for 1,536
-// rows of 1,024, this BA28).
+// rows of 1,024, this 9.4).
 __global__ void __launch_bounds__(256)
 k_batch_bf16(const void* X, int dtype, int d, const uint32_t* __restrict__ idx, int64_t R,
              int64_t Rp, int Kp, const float* __restrict__ inv_s, __nv_bfloat16* __restrict__ rows,

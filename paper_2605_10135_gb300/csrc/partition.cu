@@ -3,7 +3,8 @@
 //
 //  distances         : d32 = FP32 squared distance with the terms added in index
 //                      order, unfused (the oracle's definition).  Up to 32
-//                      centroids every d32 is computed; with more, the tensor cores screen them first: a tile query keeps the
+//                      centroids every d32 is computed; with more, the tensor
+//                      cores screen them first: a tile query keeps the
 //                      min(C, r + 6) centroids of smallest tile key per vector,
 //                      and d32 is computed for those only.  The result equals the
 //                      full d32 scan unless more than 6 other centroids lie within
@@ -313,7 +314,7 @@ __global__ void __launch_bounds__(1024)
     __shared__ int wcnt[2][32];
     const int c = blockIdx.x;
     const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
-    // S < 2^32: 32-bit sums of each warp, then over the warps in 64 bits
+    // the counts before c: 64-bit sums of each warp, then over the warps
     __shared__ unsigned long long base_s;
     if (threadIdx.x == 0) base_s = 0;
     __syncthreads();
