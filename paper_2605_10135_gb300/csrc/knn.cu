@@ -307,15 +307,13 @@ __device__ __forceinline__ bool bound_keeps(const Bound& T, uint64_t v, const ui
 // lane; n > maxkeep >= kp), exactly kp when maxkeep == kp.  Each step counts the keys at
 // or below three pivots (10 bits each of one warp sum, so all lanes return the same
 // value): two around the place where the wanted rank falls if the keys between lo and
-// hi are spread evenly, one in the middle of what lies above.  It stops as soon as the
-// keys at or below a pivot number kp to maxkeep: two or three steps for spread keys,
-// where halving the range of the key bits takes nine or more.  Where that place cannot be
-// computed (hi - lo beyond FP32's range, an infinite key) or eight steps were not enough
-// (ties, keys of very different size), the pivots quarter and halve the bits that are
-// left, at most 32 more steps: interpolation alone took 223 steps for 256 keys of three
-// values around zero, and with hi - lo = inf it came down by one bit a step.  Only when
-// more than maxkeep entries share the kp-th key are their global ids searched (then
-// exactly kp stay).
+// hi are spread evenly, and the middle of the key bits between them.  It stops as soon as
+// the keys at or below a pivot number kp to maxkeep: two or three steps for spread keys,
+// where halving the range of the key bits takes nine or more.  The middle pivot is what
+// ends every search, after 32 steps at most: interpolation alone took 223 steps for 256
+// keys of three values around zero, and where hi - lo passes FP32's range it came down by
+// one bit a step.  Only when more than maxkeep entries share the kp-th key are their
+// global ids searched (then exactly kp stay).
 static_assert(2 * kt::PH_MAX < 1024, "warp_select packs its counts in 10 bits each");
 template <int E>
 __device__ __forceinline__ Bound warp_select(const uint64_t (&v)[E], int n, int kp, int maxkeep,
@@ -333,20 +331,15 @@ __device__ __forceinline__ Bound warp_select(const uint64_t (&v)[E], int n, int 
     // invariant: #{key <= hi} = chi >= kp, #{key < lo} = clo < kp
     uint32_t lo = kmin, hi = kmax;
     int chi = n, clo = 0;
-    int interp = 8;
     while (chi > maxkeep && lo < hi) {
-        // pivots lie in [lo, hi); interpolated on the key values (on their bits a range
-        // across zero is exponential), the last one halves the bits that are left
+        // all pivots lie in [lo, hi); two are interpolated on the key values (on their bits a
+        // range across zero is exponential), in any order with the third
         const float f = (0.5f * (float)(kp + maxkeep) - (float)clo) / (float)(chi - clo);
         const float flo = ord2f(lo), fw = ord2f(hi) - flo;
         uint32_t p1 = f2ord(fmaf(0.8f * f, fw, flo)), p2 = f2ord(fmaf(1.2f * f, fw, flo));
-        if (__builtin_expect(--interp < 0 || !(fw < INFINITY), 0)) {
-            p1 = lo + ((hi - lo) >> 2);
-            p2 = lo + ((hi - lo) >> 1);
-        }
         p1 = p1 < lo ? lo : p1 > hi - 1 ? hi - 1 : p1;
         p2 = p2 < p1 ? p1 : p2 > hi - 1 ? hi - 1 : p2;
-        const uint32_t p3 = hi - 1 - ((hi - 1 - p2) >> 1);
+        const uint32_t p3 = lo + ((hi - lo) >> 1);
         uint32_t c = 0;
 #pragma unroll
         for (int e = 0; e < E; ++e) {
@@ -355,10 +348,9 @@ __device__ __forceinline__ Bound warp_select(const uint64_t (&v)[E], int n, int 
         }
         c = __reduce_add_sync(FULL, c);
         const int c1 = c & 1023, c2 = (c >> 10) & 1023, c3 = c >> 20;
-        if (c1 >= kp) { hi = p1; chi = c1; }
-        else if (c2 >= kp) { lo = p1 + 1; clo = c1; hi = p2; chi = c2; }
-        else if (c3 >= kp) { lo = p2 + 1; clo = c2; hi = p3; chi = c3; }
-        else { lo = p3 + 1; clo = c3; }
+        if (c2 >= kp) { hi = p2; chi = c2; } else { lo = p2 + 1; clo = c2; }
+        if (c1 >= kp) { hi = p1; chi = c1; } else if (p1 >= lo) { lo = p1 + 1; clo = c1; }
+        if (c3 >= kp) { if (p3 < hi) { hi = p3; chi = c3; } } else if (p3 >= lo) { lo = p3 + 1; clo = c3; }
     }
     Bound T;
     T.key = hi;
